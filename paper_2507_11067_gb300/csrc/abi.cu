@@ -79,6 +79,68 @@ bool encode_tmap_4d(CUtensorMap *map, const float *base, int64_t X, int64_t Y, i
     return r == CUDA_SUCCESS;
 }
 
+// ------------------------------------------------------- launch shapes
+cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t smem, Slots *out, size_t limit)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool cached = dev >= 0 && dev < SlotCache::kDevs;
+    if (const uint32_t w = cached ? cache.v[dev].load(std::memory_order_acquire) : 0u) {
+        *out = Slots{(int)(w >> 8), (int)(w & 255u)};
+        return cudaSuccess;
+    }
+    int sms = 0, per_sm = 0;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit > smem ? limit : smem));
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    if (e != cudaSuccess) return e;
+    if (sms < 1 || per_sm < 1 || per_sm > 255) return cudaErrorInvalidConfiguration;
+    *out = Slots{sms, per_sm};
+    if (cached) cache.v[dev].store((uint32_t)sms << 8 | (uint32_t)per_sm, std::memory_order_release);
+    return cudaSuccess;
+}
+
+// A CTA's march takes (planes + halo) steps.  An SM runs the CTAs of its
+// first 256 threads in about the time of one (two warps per scheduler; a lone
+// CTA's plane step is latency: 0.49 us for the radius-4 star, 0.23 us per
+// step and SM when four share it), and beyond that the steps share the SM.
+// So the time of a launch is about (t + halo) x the busiest SM's load, and
+// the chunk t is the one that makes it least, among those that give an SM 1,
+// 2, ... of its CTA slots and two and three full waves.  A grid whose tuned
+// chunks fill four waves or more keeps them: there the balance gains nothing
+// and more halo planes would be read.
+int z_chunk(const Slots &sl, int64_t cols, int64_t nz, int halo, int tz, int threads)
+{
+    if (cols < 1 || nz < 1) return tz;
+    const int64_t slots = (int64_t)sl.sms * sl.per_sm;
+    const double alone = threads < 256 ? 256 / threads : 1;
+    const auto cost = [&](int64_t t) {
+        const int64_t c = cols * ((nz + t - 1) / t);
+        const double n = c <= slots ? (double)((c + sl.sms - 1) / sl.sms) : (double)c / sl.sms + 0.5 * sl.per_sm;
+        return (double)(t + halo) * (n > alone ? n : alone);
+    };
+    if (tz > nz) tz = (int)nz;
+    if (cols * ((nz + tz - 1) / tz) >= 4 * slots) return tz;
+    int64_t best = tz;
+    double least = cost(tz);
+    const auto consider = [&](int64_t ctas) {
+        const int64_t k = ctas / cols;  // chunks per column
+        if (k < 1) return;
+        const int64_t t = (nz + k - 1) / k;
+        if (t > tz) return;             // the tuned chunk is the longest
+        const double c = cost(t);
+        if (c < least) {
+            least = c;
+            best = t;
+        }
+    };
+    for (int n = 1; n <= sl.per_sm; ++n) consider((int64_t)sl.sms * n);
+    consider(2 * slots);
+    consider(3 * slots);
+    return (int)best;
+}
+
 // ------------------------------------------------------- variant table
 // Registered variants (mms_set_variant): kUnset = none registered (the
 // built-in table below decides), kCleared = explicitly none, else the variant.

@@ -773,11 +773,14 @@ cudaError_t tti_deriv_r(const WaveGeo &g, const TtiCoef &cf, const float *f, con
     if (!encode_tmap_4d(&tf, f, X, Y, Z, g.nshots, g.py, g.pz, g.ss, G::BX, G::BY, 1))
         return cudaErrorInvalidValue;
     auto kern = tti_deriv_kernel<R, kTtiTX, kTtiTY, MODE>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::SMEM);
+    static SlotCache cache;
+    Slots sl;
+    cudaError_t e = kernel_slots(cache, reinterpret_cast<const void *>(kern), G::NT, T::SMEM, &sl);
     if (e != cudaSuccess) return e;
-    const int tz = kTtiTZ;
+    const int tiles_x = (g.nx + kTtiTX - 1) / kTtiTX, tiles_y = (g.ny + kTtiTY - 1) / kTtiTY;
+    const int tz = z_chunk(sl, (int64_t)tiles_x * tiles_y * g.nshots, g.nz, 2 * R, kTtiTZ, G::NT);
     const int nzc = (g.nz + tz - 1) / tz;
-    const dim3 grid((g.nx + kTtiTX - 1) / kTtiTX, (g.ny + kTtiTY - 1) / kTtiTY, nzc * g.nshots);
+    const dim3 grid(tiles_x, tiles_y, nzc * g.nshots);
     int vec = g.nx % 4 == 0 && reinterpret_cast<uintptr_t>(tilt) % 16 == 0 &&
               reinterpret_cast<uintptr_t>(lap) % 16 == 0 && reinterpret_cast<uintptr_t>(h1) % 16 == 0;
     if (MODE == 2)
@@ -844,10 +847,14 @@ cudaError_t vti_launch(const WaveGeo &g, const StarCoef &cf, int tz, const float
         !encode_tmap_4d(&tm.vc, vcur, X, Y, Z, g.nshots, g.py, g.pz, g.ss, I::BXI, TY, 1))
         return cudaErrorInvalidValue;
     auto kern = vti_fwd_kernel<R, TX, TY, S>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)V::SMEM);
+    static SlotCache cache;
+    Slots sl;
+    cudaError_t e = kernel_slots(cache, reinterpret_cast<const void *>(kern), G::NT, V::SMEM, &sl);
     if (e != cudaSuccess) return e;
+    const int tiles_x = (g.nx + TX - 1) / TX, tiles_y = (g.ny + TY - 1) / TY;
+    tz = z_chunk(sl, (int64_t)tiles_x * tiles_y * g.nshots, g.nz, 2 * R, tz, G::NT);
     const int nzc = (g.nz + tz - 1) / tz;
-    const dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, nzc * g.nshots);
+    const dim3 grid(tiles_x, tiles_y, nzc * g.nshots);
     const int vec = (R % 4 == 0) && g.py % 4 == 0 && g.pz % 4 == 0 && g.ss % 4 == 0 &&
                     reinterpret_cast<uintptr_t>(hnext) % 16 == 0 && reinterpret_cast<uintptr_t>(vnext) % 16 == 0;
     kern<<<grid, G::NT, V::SMEM, st>>>(tm, cf, g, hnext, vnext, amp, rec, tz, nzc, vec, device_error_word());

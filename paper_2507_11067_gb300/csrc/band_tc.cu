@@ -838,19 +838,6 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
     }
 }
 
-int g_num_sms = 0;
-
-int num_sms()
-{
-    if (g_num_sms == 0) {
-        int dev = 0, n = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        g_num_sms = n > 0 ? n : 152;
-    }
-    return g_num_sms;
-}
-
 // What one launch computes: the band weights (box: (2r+1)^3; planar and
 // star: the (2r+1)^2 in-plane set), the star's z weights, where the staged
 // planes start, and where the results go.
@@ -879,7 +866,16 @@ cudaError_t launch_r(const Sweep &s, const CUtensorMap &map, int nzt, const Laun
     a.nz = (int)s.nz;
     const uintptr_t ob = reinterpret_cast<uintptr_t>(L.out);
     a.vec = (L.opy % 4 == 0 && L.opz % 4 == 0 && ob % 16 == 0) ? 4 : (L.opy % 2 == 0 && L.opz % 2 == 0 && ob % 8 == 0) ? 2 : 1;
-    const int64_t tx = (s.nx + C::TX - 1) / C::TX, ty = (s.ny + C::TY - 1) / C::TY, tz = (s.nz + nzt - 1) / nzt;
+    auto kern = band_tc_kernel<R, PREC, MODE>;
+    static SlotCache cache;
+    Slots sl;
+    cudaError_t e = kernel_slots(cache, reinterpret_cast<const void *>(kern), C::NT, C::SMEM, &sl);
+    if (e != cudaSuccess) return e;
+    // persistent: one CTA per SM, two for the dual configuration
+    sl.per_sm = C::DUAL ? 2 : 1;
+    const int64_t tx = (s.nx + C::TX - 1) / C::TX, ty = (s.ny + C::TY - 1) / C::TY;
+    nzt = z_chunk(sl, tx * ty, s.nz, 2 * C::RZ, nzt, C::NT);
+    const int64_t tz = (s.nz + nzt - 1) / nzt;
     if (tx * ty * tz > (int64_t)1 << 30) return cudaErrorInvalidValue;
     a.tiles_x = (int)tx;
     a.tiles_y = (int)ty;
@@ -893,11 +889,7 @@ cudaError_t launch_r(const Sweep &s, const CUtensorMap &map, int nzt, const Laun
     CUtensorMap omap{};
     a.tstore = C::TSTORE && a.vec == 4 &&
                encode_tmap_3d(&omap, L.out, s.nx, s.ny, s.nz, L.opy, L.opz, C::TSTORE ? C::TXO : 4, C::TY, 1);
-    auto kern = band_tc_kernel<R, PREC, MODE>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    if (e != cudaSuccess) return e;
-    // persistent: one CTA per SM, two for the dual configuration
-    const int slots = num_sms() * (C::DUAL ? 2 : 1);
+    const int slots = sl.sms * sl.per_sm;
     const int grid = a.tiles < slots ? a.tiles : slots;
     kern<<<grid, C::NT, C::SMEM, s.stream>>>(map, omap, cf, a, device_error_word());
     return cudaGetLastError();

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/mms.h"
 
 namespace mms {
@@ -80,6 +82,24 @@ bool encode_tmap_3d(CUtensorMap *map, const float *base, int64_t X, int64_t Y, i
 // The same over nw stacked grids `pw` elements apart, box depth 1 in w.
 bool encode_tmap_4d(CUtensorMap *map, const float *base, int64_t X, int64_t Y, int64_t Z,
                     int64_t W, int64_t py, int64_t pz, int64_t pw, int bx, int by, int bz);
+
+// What one kernel instance can keep resident on a device, asked once per
+// device (with its dynamic shared-memory limit set to `limit`, by default
+// `smem`; launches of one kernel with several sizes pass the largest): the SM
+// count and the CTAs of `threads` threads and `smem` bytes one SM holds.  One
+// static cache per kernel instance and size; concurrent first calls compute
+// the same values.
+struct SlotCache {
+    static constexpr int kDevs = 64;
+    std::atomic<uint32_t> v[kDevs];  // SMs << 8 | CTAs per SM, 0 = not asked yet
+};
+struct Slots { int sms = 0, per_sm = 0; };
+cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t smem, Slots *out, size_t limit = 0);
+
+// Planes per z chunk of a kernel whose CTAs each march one chunk of one of
+// `cols` columns (reading `halo` extra planes), given the kernel's tuned
+// chunk `tz`.
+int z_chunk(const Slots &sl, int64_t cols, int64_t nz, int halo, int tz, int threads);
 
 }  // namespace mms
 

@@ -212,11 +212,13 @@ cudaError_t launch_tiled(const Sweep &sw, const CUtensorMap &tmap, const Coef &c
 {
     using G = Geom<R, TX, TY, PY, S>;
     auto kern = sweep_cc_kernel<R, TX, TY, PY, S, BOX, ROTQ, ONEW, Coef>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)G::SMEM);
+    static SlotCache cache;
+    Slots sl;
+    cudaError_t e = kernel_slots(cache, reinterpret_cast<const void *>(kern), G::NT, G::SMEM, &sl);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)((sw.nx + TX - 1) / TX), (unsigned)((sw.ny + TY - 1) / TY),
-                    (unsigned)((sw.nz + tz - 1) / tz));
+    const int64_t tiles_x = (sw.nx + TX - 1) / TX, tiles_y = (sw.ny + TY - 1) / TY;
+    tz = z_chunk(sl, tiles_x * tiles_y, sw.nz, 2 * R, tz, G::NT);
+    const dim3 grid((unsigned)tiles_x, (unsigned)tiles_y, (unsigned)((sw.nz + tz - 1) / tz));
     const int vec = ((sw.opy % 4) == 0 && (sw.opz % 4) == 0 &&
                      (reinterpret_cast<uintptr_t>(sw.out) % 16) == 0)
                         ? 1

@@ -722,38 +722,26 @@ cudaError_t fwd_r(const WaveGeo &g, const StarCoef &cf, const float *m, const fl
     const size_t smem = mode == K_ADJ_SCALED ? FA::SMEM - (gbulk ? 0 : FA::GB_BYTES)
                         : mode == K_FWD_LAP  ? FwdGeom<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_FWD_LAP>::SMEM
                                              : FwdGeom<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_FWD>::SMEM;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SlotCache caches[4];  // per form (the adjoint without and with its gradient buffers)
+    Slots sl;
+    cudaError_t e = kernel_slots(caches[mode + (gbulk ? 1 : 0)], reinterpret_cast<const void *>(kern), G::NT, smem, &sl,
+                                 mode == K_ADJ_SCALED ? FA::SMEM : smem);
     if (e != cudaSuccess) return e;
-    // z chunks of kFwdTZ planes.  The adjoint step on a grid whose CTAs fill
-    // at most one wave splits z finer, into about three waves, so that the
-    // SMs left with one CTA do not idle while the others finish two (2 x
-    // 256^3: 219 -> 207 us per step; the forward forms gained nothing).
-    const int cols = (g.nx + kFwdTX - 1) / kFwdTX * ((g.ny + kFwdTY - 1) / kFwdTY) * g.nshots;
-    int tz = kFwdTZ;
-    if (mode == K_ADJ_SCALED) {
-        // resident CTAs of this launch on the current device (cached per
-        // device, without / with the gradient buffers)
-        constexpr int kDevs = 16;
-        static int slots[kDevs][2] = {};
-        int dev = 0, sl_local = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
-        int &sl = dev >= 0 && dev < kDevs ? slots[dev][gbulk ? 1 : 0] : sl_local;
-        if (sl == 0) {
-            int sms = 0, per_sm = 0;
-            if (dev >= 0 && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, G::NT, smem) == cudaSuccess)
-                sl = sms * per_sm > 0 ? sms * per_sm : -1;
-            else
-                sl = -1;
-        }
-        if (sl > 0 && cols * ((g.nz + tz - 1) / tz) <= sl) {
-            const int k = (3 * sl + cols / 2) / cols;  // chunks per column for about three waves
-            tz = k > 0 ? (g.nz + k - 1) / k : tz;
-            if (tz < 2 * R) tz = 2 * R;
-        }
+    const int tiles_x = (g.nx + kFwdTX - 1) / kFwdTX, tiles_y = (g.ny + kFwdTY - 1) / kFwdTY;
+    const int64_t cols = (int64_t)tiles_x * tiles_y * g.nshots, slots = (int64_t)sl.sms * sl.per_sm;
+    int tz = z_chunk(sl, cols, g.nz, 2 * R, kFwdTZ, G::NT);
+    // The adjoint step on a grid whose CTAs fill most of one wave splits z
+    // finer, into about three waves, so that the SMs left with one CTA do not
+    // idle while the others finish two (2 x 256^3: 219 -> 207 us per step; the
+    // forward forms gained nothing).
+    if (mode == K_ADJ_SCALED && 2 * cols * ((g.nz + kFwdTZ - 1) / kFwdTZ) > slots &&
+        cols * ((g.nz + kFwdTZ - 1) / kFwdTZ) <= slots) {
+        const int k = (int)((3 * slots + cols / 2) / cols);  // chunks per column for about three waves
+        tz = k > 0 ? (g.nz + k - 1) / k : tz;
+        if (tz < 2 * R) tz = 2 * R;
     }
     const int nzc = (g.nz + tz - 1) / tz;
-    const dim3 grid((g.nx + kFwdTX - 1) / kFwdTX, (g.ny + kFwdTY - 1) / kFwdTY, nzc * g.nshots);
+    const dim3 grid(tiles_x, tiles_y, nzc * g.nshots);
     const int vec = (R % 4 == 0) && g.py % 4 == 0 && g.pz % 4 == 0 && g.ss % 4 == 0 &&
                     reinterpret_cast<uintptr_t>(p_next) % 16 == 0 && reinterpret_cast<uintptr_t>(lapout) % 16 == 0;
     const AdjArgs aa = adj ? *adj : AdjArgs{nullptr, nullptr, 0, 0};
@@ -784,11 +772,14 @@ cudaError_t adj_r(const WaveGeo &g, const StarCoef &cf, const float *m, const fl
         ma = ml;
     }
     auto kern = wave_adj_kernel<R, kAdjTX, kAdjTY, kAdjS, LAPIN>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A::SMEM);
+    static SlotCache cache;
+    Slots sl;
+    cudaError_t e = kernel_slots(cache, reinterpret_cast<const void *>(kern), G::NT, A::SMEM, &sl);
     if (e != cudaSuccess) return e;
-    const int tz = kAdjTZ;
+    const int tiles_x = (g.nx + kAdjTX - 1) / kAdjTX, tiles_y = (g.ny + kAdjTY - 1) / kAdjTY;
+    const int tz = z_chunk(sl, (int64_t)tiles_x * tiles_y * g.nshots, g.nz, 2 * R, kAdjTZ, G::NT);
     const int nzc = (g.nz + tz - 1) / tz;
-    const dim3 grid((g.nx + kAdjTX - 1) / kAdjTX, (g.ny + kAdjTY - 1) / kAdjTY, nzc * g.nshots);
+    const dim3 grid(tiles_x, tiles_y, nzc * g.nshots);
     // 32-byte aligned rows of four doubles: two double2 per thread
     const int gvec = g.nx % 4 == 0 && g.gss % 4 == 0 && reinterpret_cast<uintptr_t>(grad) % 32 == 0;
     kern<<<grid, G::NT, A::SMEM, st>>>(ml, mm, ma, m2, m1, cf, g, lam_prev, resid, grad, a_n ? 1 : 0,
