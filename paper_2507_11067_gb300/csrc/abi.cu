@@ -80,7 +80,7 @@ bool encode_tmap_4d(CUtensorMap *map, const float *base, int64_t X, int64_t Y, i
 }
 
 // ------------------------------------------------------- launch shapes
-cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t smem, Slots *out, size_t limit)
+cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t smem, Slots *out)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -91,7 +91,7 @@ cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t
         return cudaSuccess;
     }
     int sms = 0, per_sm = 0;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(limit > smem ? limit : smem));
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPerCta);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
     if (e != cudaSuccess) return e;
@@ -101,44 +101,49 @@ cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t
     return cudaSuccess;
 }
 
-// A CTA's march takes (planes + halo) steps.  An SM runs the CTAs of its
-// first 256 threads in about the time of one (two warps per scheduler; a lone
-// CTA's plane step is latency: 0.49 us for the radius-4 star, 0.23 us per
-// step and SM when four share it), and beyond that the steps share the SM.
-// So the time of a launch is about (t + halo) x the busiest SM's load, and
-// the chunk t is the one that makes it least, among those that give an SM 1,
-// 2, ... of its CTA slots and two and three full waves.  A grid whose tuned
-// chunks fill four waves or more keeps them: there the balance gains nothing
-// and more halo planes would be read.
+// CTAs per SM up to which another one costs an SM nothing: 256 threads are two
+// warps per scheduler, and a plane step of fewer is latency (the radius-4
+// star: 0.49 us for a lone CTA of 128 threads, 0.23 us per CTA when four
+// share the SM); and the CTAs that keep an SM busy (512 threads).
+static int free_ctas(int threads) { return threads < 256 ? 256 / threads : 1; }
+static int busy_ctas(const Slots &sl, int threads)
+{
+    const int n = (512 + threads - 1) / threads;
+    return n < sl.per_sm ? n : sl.per_sm;
+}
+
 int z_chunk(const Slots &sl, int64_t cols, int64_t nz, int halo, int tz, int threads)
 {
     if (cols < 1 || nz < 1) return tz;
-    const int64_t slots = (int64_t)sl.sms * sl.per_sm;
-    const double alone = threads < 256 ? 256 / threads : 1;
-    const auto cost = [&](int64_t t) {
-        const int64_t c = cols * ((nz + t - 1) / t);
-        const double n = c <= slots ? (double)((c + sl.sms - 1) / sl.sms) : (double)c / sl.sms + 0.5 * sl.per_sm;
-        return (double)(t + halo) * (n > alone ? n : alone);
-    };
     if (tz > nz) tz = (int)nz;
-    if (cols * ((nz + tz - 1) / tz) >= 4 * slots) return tz;
-    int64_t best = tz;
-    double least = cost(tz);
-    const auto consider = [&](int64_t ctas) {
-        const int64_t k = ctas / cols;  // chunks per column
-        if (k < 1) return;
-        const int64_t t = (nz + k - 1) / k;
-        if (t > tz) return;             // the tuned chunk is the longest
-        const double c = cost(t);
-        if (c < least) {
-            least = c;
-            best = t;
-        }
+    const int busy = busy_ctas(sl, threads), alone = free_ctas(threads);
+    if (cols * ((nz + tz - 1) / tz) >= (int64_t)sl.sms * busy) return tz;
+    const auto cost = [&](int64_t t) {
+        const int64_t n = (cols * ((nz + t - 1) / t) + sl.sms - 1) / sl.sms;
+        return (t + halo) * (n > alone ? n : alone);
     };
-    for (int n = 1; n <= sl.per_sm; ++n) consider((int64_t)sl.sms * n);
-    consider(2 * slots);
-    consider(3 * slots);
+    int64_t best = tz;
+    for (int n = 1; n <= busy; ++n) {
+        const int64_t k = (int64_t)sl.sms * n / cols;  // chunks per column
+        if (k < 1) continue;
+        const int64_t t = (nz + k - 1) / k;
+        if (t <= tz && cost(t) < cost(best)) best = t;
+    }
     return (int)best;
+}
+
+March plan_march(const Slots &sl, int64_t tiles_x, int64_t tiles_y, int nshots, int64_t nz, int halo, int tz,
+                 int threads, size_t *smem, int64_t *ctas)
+{
+    const int64_t cols = tiles_x * tiles_y * nshots;
+    tz = z_chunk(sl, cols, nz, halo, tz, threads);
+    *ctas = cols * ((nz + tz - 1) / tz);
+    const int64_t n = (*ctas + sl.sms - 1) / sl.sms;  // CTAs per SM, spread evenly
+    if (n < sl.per_sm) {
+        const size_t least = kSmemPerSm / (size_t)(n + 1) - kSmemReserved + 16;  // n + 1 of these do not fit
+        if (*smem < least) *smem = least < kSmemPerCta ? least : kSmemPerCta;
+    }
+    return March{(int)tiles_x, (int)tiles_y, nshots, tz};
 }
 
 // ------------------------------------------------------- variant table

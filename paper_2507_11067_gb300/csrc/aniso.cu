@@ -58,8 +58,8 @@ template <int R, int TX, int TY, int S>
 __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT)
     vti_fwd_kernel(const __grid_constant__ VtiMaps tm, const __grid_constant__ StarCoef cf,
                    const __grid_constant__ WaveGeo geo, float *__restrict__ hnext, float *__restrict__ vnext,
-                   const float *__restrict__ amp, float *__restrict__ rec, int tz, int nzc, int vec,
-                   unsigned *err)
+                   const float *__restrict__ amp, float *__restrict__ rec,
+                   const __grid_constant__ March march, int vec, unsigned *err)
 {
     using G = Geom<R, TX, TY, 1, S>;
     using V = VtiGeom<R, TX, TY, S>;
@@ -73,14 +73,26 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT)
 
     const int tid = threadIdx.x;
     const int tx = tid % G::NTX, ty = tid / G::NTX;
-    const int sh = blockIdx.z / nzc, zc = blockIdx.z % nzc;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, zb = zc * tz;
-    const int nzt = min(tz, geo.nz - zb);
+    if (tid == 0) {
+        ptx::prefetch_tmap(&tm.h);
+        ptx::prefetch_tmap(&tm.v);
+        ptx::prefetch_tmap(&tm.rho);
+        ptx::prefetch_tmap(&tm.mv);
+        ptx::prefetch_tmap(&tm.hp);
+        ptx::prefetch_tmap(&tm.vp);
+#pragma unroll
+        for (int s = 0; s < S; ++s) ptx::mbar_init(&full[s], 1);
+        ptx::fence_mbar_init();
+        abort_flag = 0;
+    }
+    const Leg leg = leg_of(march);
+    const int sh = leg.shot, x0 = leg.tx * TX, y0 = leg.ty * TY, zb = leg.zc * march.tz;
+    const int nzt = min(march.tz, geo.nz - zb);
     const int P = nzt + 2 * R;
     const int gx = x0 + 4 * tx;
     const int sx = geo.src[sh][0], sy = geo.src[sh][1], sz = geo.src[sh][2];
-
-    auto issue = [&](int j, int s) {
+    auto issue = [&](int j) {
+        const int s = j % S;
         float *st = stages + (size_t)s * V::STAGE;
         const bool centre = j >= R && j < R + nzt;  // an output plane of this chunk
         const bool done = j >= 2 * R;               // completes output plane j - 2R
@@ -100,21 +112,9 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT)
             ptx::tma_load_4d(st + V::OFF_VC, &tm.vc, xs, y0 + R, zp, sh, &full[s]);
         }
     };
-    if (tid == 0) {
-        ptx::prefetch_tmap(&tm.h);
-        ptx::prefetch_tmap(&tm.v);
-        ptx::prefetch_tmap(&tm.rho);
-        ptx::prefetch_tmap(&tm.mv);
-        ptx::prefetch_tmap(&tm.hp);
-        ptx::prefetch_tmap(&tm.vp);
-#pragma unroll
-        for (int s = 0; s < S; ++s) ptx::mbar_init(&full[s], 1);
-        ptx::fence_mbar_init();
-        abort_flag = 0;
-    }
     __syncthreads();
     if (tid == 0)
-        for (int j = 0; j < S && j < P; ++j) issue(j, j);
+        for (int j = 0; j < S && j < P; ++j) issue(j);
 
     float gxs[4];
 #pragma unroll
@@ -122,11 +122,11 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT)
     const float gys = sponge(y0 + ty, geo.ny, geo.sponge_w, geo.sponge_a);
 
     // qh: rho Lh sigma_H + Lz sigma_V; qv: Lh sigma_V / rho + Lz sigma_H
-    float qh[W][4], qv[W][4];
+    f2 qh[W][2], qv[W][2];
 #pragma unroll
     for (int kk = 0; kk < W; ++kk)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) qh[kk][k] = qv[kk][k] = 0.f;
+        for (int h = 0; h < 2; ++h) qh[kk][h] = qv[kk][h] = zero2();
 
     const float samp = amp[sh];
     const int64_t shot_off = (int64_t)sh * geo.ss;
@@ -138,52 +138,48 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT)
         float mv[4], rz[4], hp[4], vp[4], hc[4], vc[4];
         if (ptx::mbar_wait_bounded(&full[s], (uint32_t)(j / S) & 1u, err)) {
             const float *ph = st, *pv = st + V::OFF_V;
-            float ch[4], cv[4];
-            load_center<R>(ph + (ty + R) * G::BX + 4 * tx, ch);
-            load_center<R>(pv + (ty + R) * G::BX + 4 * tx, cv);
+            f2 ch[2], cv[2];
+            load_center2<R>(ph + (ty + R) * G::BX + 4 * tx, ch);
+            load_center2<R>(pv + (ty + R) * G::BX + 4 * tx, cv);
             // z part: this plane is offset R - kk from the output plane of slot kk
 #pragma unroll
-            for (int kk = 0; kk < W; ++kk)
+            for (int kk = 0; kk < W; ++kk) {
+                const f2 wz = pair(cf.c[2 * W + 2 * R - kk]);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float wz = cf.c[2 * W + 2 * R - kk];
-                    qh[kk][k] = fmaf(wz, cv[k], qh[kk][k]);
-                    qv[kk][k] = fmaf(wz, ch[k], qv[kk][k]);
+                for (int h = 0; h < 2; ++h) {
+                    qh[kk][h] = fma2(wz, cv[h], qh[kk][h]);
+                    qv[kk][h] = fma2(wz, ch[h], qv[kk][h]);
                 }
+            }
             if (centre) {
                 float rc[4];
                 load_center<I::OFF>(st + V::OFF_RC + ty * I::BXI + 4 * tx, rc);
                 float wh[4 * G::NV], wv[4 * G::NV];
                 load_row<G::NV>(ph + (ty + R) * G::BX + 4 * tx, wh);
                 load_row<G::NV>(pv + (ty + R) * G::BX + 4 * tx, wv);
-                float lh[4], lv[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    lh[k] = 0.f;
-                    lv[k] = 0.f;
-#pragma unroll
-                    for (int d = -R; d <= R; ++d) {
-                        lh[k] = fmaf(cf.c[d + R], wh[k + R + d], lh[k]);
-                        lv[k] = fmaf(cf.c[d + R], wv[k + R + d], lv[k]);
-                    }
-                }
+                f2 lh[2] = {zero2(), zero2()}, lv[2] = {zero2(), zero2()};
+                line_x<R>(cf.c, wh, lh);
+                line_x<R>(cf.c, wv, lv);
 #pragma unroll
                 for (int d = -R; d <= R; ++d) {
-                    float ah[4], av[4];
-                    load_center<R>(ph + (ty + R + d) * G::BX + 4 * tx, ah);
-                    load_center<R>(pv + (ty + R + d) * G::BX + 4 * tx, av);
+                    f2 ah[2], av[2];
+                    load_center2<R>(ph + (ty + R + d) * G::BX + 4 * tx, ah);
+                    load_center2<R>(pv + (ty + R + d) * G::BX + 4 * tx, av);
+                    const f2 wy = pair(cf.c[W + d + R]);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        lh[k] = fmaf(cf.c[W + d + R], ah[k], lh[k]);
-                        lv[k] = fmaf(cf.c[W + d + R], av[k], lv[k]);
+                    for (int h = 0; h < 2; ++h) {
+                        lh[h] = fma2(wy, ah[h], lh[h]);
+                        lv[h] = fma2(wy, av[h], lv[h]);
                     }
                 }
+                // rho > 0 inside the grid; the guard keeps lanes past the edge finite
+                float inv[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    // rho > 0 inside the grid; the guard keeps lanes past the edge finite
-                    const float inv = rc[k] != 0.f ? 1.f / rc[k] : 0.f;
-                    qh[R][k] = fmaf(rc[k], lh[k], qh[R][k]);
-                    qv[R][k] = fmaf(inv, lv[k], qv[R][k]);
+                for (int k = 0; k < 4; ++k) inv[k] = rc[k] != 0.f ? 1.f / rc[k] : 0.f;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    qh[R][h] = fma2(pair(rc[2 * h], rc[2 * h + 1]), lh[h], qh[R][h]);
+                    qv[R][h] = fma2(pair(inv[2 * h], inv[2 * h + 1]), lv[h], qv[R][h]);
                 }
             }
             if (zo >= 0) {
@@ -200,20 +196,25 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT)
         }
         __syncthreads();
         if (abort_flag) return;
-        if (tid == 0 && j + S < P) issue(j + S, s);
+        if (tid == 0 && j + S < P) issue(j + S);
         if (zo >= 0) {
             const int z = zb + zo;
             const int y = y0 + ty;
             const float gzv = sponge(z, geo.nz, geo.sponge_w, geo.sponge_a);
             if (y < geo.ny && gx < geo.nx) {
                 const int64_t mp = (int64_t)(z + R) * geo.pz + (int64_t)(y + R) * geo.py + (gx + R);
-                float rh[4], rv[4];
+                float rh[4], rv[4], ah[4], av[4];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    unpair(qh[0][h], ah[2 * h], ah[2 * h + 1]);
+                    unpair(qv[0][h], av[2 * h], av[2 * h + 1]);
+                }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const float g = gxs[k] * gys * gzv;
                     const bool at_src = gx + k == sx && y == sy && z == sz;
-                    float a = 2.f * hc[k] + mv[k] * qh[0][k] - g * hp[k];
-                    float b = 2.f * vc[k] + (mv[k] * rz[k]) * qv[0][k] - g * vp[k];
+                    float a = 2.f * hc[k] + mv[k] * ah[k] - g * hp[k];
+                    float b = 2.f * vc[k] + (mv[k] * rz[k]) * av[k] - g * vp[k];
                     if (at_src) {
                         a += samp;
                         b += samp;
@@ -244,12 +245,12 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT)
 #pragma unroll
         for (int kk = 0; kk < W - 1; ++kk)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                qh[kk][k] = qh[kk + 1][k];
-                qv[kk][k] = qv[kk + 1][k];
+            for (int h = 0; h < 2; ++h) {
+                qh[kk][h] = qh[kk + 1][h];
+                qv[kk][h] = qv[kk + 1][h];
             }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) qh[W - 1][k] = qv[W - 1][k] = 0.f;
+        for (int h = 0; h < 2; ++h) qh[W - 1][h] = qv[W - 1][h] = zero2();
     }
 }
 
@@ -304,8 +305,8 @@ __global__ void vti_model_kernel(WaveGeo geo, const float *__restrict__ vp, cons
 // and the damped leapfrog update, source and receivers of the acoustic step.
 
 struct TtiCoef {
-    float w2[2 * kMaxR + 1];
-    float w1[2 * kMaxR + 1];
+    W2 w2[2 * kMaxR + 1];
+    W2 w1[2 * kMaxR + 1];
 };
 
 // MODE 0: p or q pass, tilt by plain loads (rows TMA cannot stage);
@@ -349,58 +350,79 @@ struct TtiFused {
     float *rec;
 };
 
+// acc (points 0..3) = the first derivative along x of a window row: taps
+// -d and d together, d ascending, paired where the columns allow it (line_x).
+template <int R>
+__device__ __forceinline__ void deriv_x(const W2 *w1, const float *row, f2 (&acc)[2])
+{
+    acc[0] = acc[1] = zero2();
+#pragma unroll
+    for (int d = 1; d <= R; ++d) {
+        if ((R + d) % 2 == 0) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                acc[h] = fma2(pair(w1[R - d]), pair(row[2 * h + R - d], row[2 * h + R - d + 1]), acc[h]);
+                acc[h] = fma2(pair(w1[R + d]), pair(row[2 * h + R + d], row[2 * h + R + d + 1]), acc[h]);
+            }
+        } else {
+            const float a = w1[R - d].lo, b = w1[R + d].lo;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                acc[h].x = fmaf(b, row[2 * h + R + d], fmaf(a, row[2 * h + R - d], acc[h].x));
+                acc[h].y = fmaf(b, row[2 * h + 1 + R + d], fmaf(a, row[2 * h + 1 + R - d], acc[h].y));
+            }
+        }
+    }
+}
+
 // The arriving plane's contributions to the z queues: centre value (f_zz),
 // D_x f (f_xz) and D_y f (f_yz), each weighted for the slot's offset.
 template <int R, int NV, int BX, int NTX>
 __device__ __forceinline__ void tti_arrive(const float *pl, const TtiCoef &cf, int tx, int ty,
-                                           float (&qzz)[2 * R + 1][4], float (&qxz)[2 * R + 1][4],
-                                           float (&qyz)[2 * R + 1][4], float *dyrow)
+                                           f2 (&qzz)[2 * R + 1][2], f2 (&qxz)[2 * R + 1][2],
+                                           f2 (&qyz)[2 * R + 1][2], float *dyrow)
 {
     constexpr int W = 2 * R + 1;
     float win[4 * NV];
     load_row<NV>(pl + (ty + R) * BX + 4 * tx, win);
-    float dx[4], dy[4], c0[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        c0[k] = win[k + R];
-        dx[k] = 0.f;
-#pragma unroll
-        for (int d = 1; d <= R; ++d)
-            dx[k] = fmaf(cf.w1[R + d], win[k + R + d], fmaf(cf.w1[R - d], win[k + R - d], dx[k]));
-        dy[k] = 0.f;
-    }
+    f2 dx[2], dy[2] = {zero2(), zero2()};
+    const f2 c0[2] = {pair(win[R], win[R + 1]), pair(win[R + 2], win[R + 3])};
+    deriv_x<R>(cf.w1, win, dx);
 #pragma unroll
     for (int d = -R; d <= R; ++d) {
         if (d == 0) continue;
-        float a[4];
-        load_center<R>(pl + (ty + R + d) * BX + 4 * tx, a);
+        f2 a[2];
+        load_center2<R>(pl + (ty + R + d) * BX + 4 * tx, a);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) dy[k] = fmaf(cf.w1[R + d], a[k], dy[k]);
+        for (int h = 0; h < 2; ++h) dy[h] = fma2(pair(cf.w1[R + d]), a[h], dy[h]);
     }
     // D_y f into the ring row at the plane's column indices; the x-halo
     // columns that f_xy's window reaches (R on each side) take one thread
     // each, the row's first 2R, so that a warp runs the halo sums once
     // instead of R times on two threads
+    float dyv[4];
+    unpair(dy[0], dyv[0], dyv[1]);
+    unpair(dy[1], dyv[2], dyv[3]);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) dyrow[4 * tx + R + k] = dy[k];
+    for (int k = 0; k < 4; ++k) dyrow[4 * tx + R + k] = dyv[k];
     static_assert(NTX >= 2 * R, "a thread per x-halo column");
     if (tx < 2 * R) {
         const int c = tx < R ? tx : 4 * NTX + tx;  // 0 .. R-1, then 4 NTX + R .. 4 NTX + 2R - 1
         float v = 0.f;
 #pragma unroll
         for (int d = -R; d <= R; ++d)
-            if (d != 0) v = fmaf(cf.w1[R + d], pl[(ty + R + d) * BX + c], v);
+            if (d != 0) v = fmaf(cf.w1[R + d].lo, pl[(ty + R + d) * BX + c], v);
         dyrow[c] = v;
     }
 #pragma unroll
     for (int kk = 0; kk < W; ++kk)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int h = 0; h < 2; ++h) {
             const int d = R - kk;  // offset of this plane from slot kk's output plane
-            qzz[kk][k] = fmaf(cf.w2[R + d], c0[k], qzz[kk][k]);
+            qzz[kk][h] = fma2(pair(cf.w2[R + d]), c0[h], qzz[kk][h]);
             if (d != 0) {
-                qxz[kk][k] = fmaf(cf.w1[R + d], dx[k], qxz[kk][k]);
-                qyz[kk][k] = fmaf(cf.w1[R + d], dy[k], qyz[kk][k]);
+                qxz[kk][h] = fma2(pair(cf.w1[R + d]), dx[h], qxz[kk][h]);
+                qyz[kk][h] = fma2(pair(cf.w1[R + d]), dy[h], qyz[kk][h]);
             }
         }
 }
@@ -414,26 +436,27 @@ __device__ __forceinline__ void tti_centre(const float *pc, const float *dyrow, 
     float w[4 * NV], v[4 * NV];
     load_row<NV>(pc + (ty + R) * BX + 4 * tx, w);
     load_row<NV>(dyrow + 4 * tx, v);
+    f2 xx[2] = {zero2(), zero2()}, yy[2], xy[2];
+    line_x<R>(cf.w2, w, xx);
+    deriv_x<R>(cf.w1, v, xy);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        ctr[k] = w[k + R];
-        fxx[k] = 0.f;
-        fxy[k] = 0.f;
-#pragma unroll
-        for (int a = -R; a <= R; ++a) fxx[k] = fmaf(cf.w2[R + a], w[k + R + a], fxx[k]);
-#pragma unroll
-        for (int a = 1; a <= R; ++a)
-            fxy[k] = fmaf(cf.w1[R + a], v[k + R + a], fmaf(cf.w1[R - a], v[k + R - a], fxy[k]));
-        fyy[k] = cf.w2[R] * w[k + R];
-    }
+    for (int h = 0; h < 2; ++h) yy[h] = mul2(pair(cf.w2[R]), pair(w[R + 2 * h], w[R + 2 * h + 1]));
 #pragma unroll
     for (int b = -R; b <= R; ++b) {
         if (b == 0) continue;
-        float a[4];
-        load_center<R>(pc + (ty + R + b) * BX + 4 * tx, a);
+        f2 a[2];
+        load_center2<R>(pc + (ty + R + b) * BX + 4 * tx, a);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) fyy[k] = fmaf(cf.w2[R + b], a[k], fyy[k]);
+        for (int h = 0; h < 2; ++h) yy[h] = fma2(pair(cf.w2[R + b]), a[h], yy[h]);
     }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        unpair(xx[h], fxx[2 * h], fxx[2 * h + 1]);
+        unpair(yy[h], fyy[2 * h], fyy[2 * h + 1]);
+        unpair(xy[h], fxy[2 * h], fxy[2 * h + 1]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) ctr[k] = w[k + R];
 }
 
 __device__ __forceinline__ float tti_h1(float nx, float ny, float nz, float fxx, float fyy, float fzz, float fxy,
@@ -455,7 +478,7 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, R + 3>::NT)
     tti_deriv_kernel(const __grid_constant__ CUtensorMap tf, const __grid_constant__ TtiCoef cf,
                      const __grid_constant__ WaveGeo geo, const float *__restrict__ tilt, TtiDense dn,
                      float *__restrict__ lap, float *__restrict__ h1, const __grid_constant__ TtiFused fu,
-                     int tz, int nzc, int vec, unsigned *err)
+                     const __grid_constant__ March march, int vec, unsigned *err)
 {
     using T = TtiGeom<R, TX, TY, MODE>;
     using G = typename T::G;
@@ -474,13 +497,22 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, R + 3>::NT)
 
     const int tid = threadIdx.x;
     const int tx = tid % G::NTX, ty = tid / G::NTX;
-    const int sh = blockIdx.z / nzc, zc = blockIdx.z % nzc;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, zb = zc * tz;
-    const int nzt = min(tz, geo.nz - zb);
-    const int P = nzt + 2 * R;
-    const int gx = x0 + 4 * tx, y = y0 + ty;
     const int64_t npts = (int64_t)geo.nz * dn.sz;  // one dense field
 
+    if (tid == 0) {
+        ptx::prefetch_tmap(&tf);
+#pragma unroll
+        for (int s = 0; s < S; ++s) ptx::mbar_init(&full[s], 1);
+#pragma unroll
+        for (int c = 0; c < T::CRING; ++c) ptx::mbar_init(&cfull[c], 1);
+        ptx::fence_mbar_init();
+        abort_flag = 0;
+    }
+    const Leg leg = leg_of(march);
+    const int sh = leg.shot, x0 = leg.tx * TX, y0 = leg.ty * TY, zb = leg.zc * march.tz;
+    const int nzt = min(march.tz, geo.nz - zb);
+    const int P = nzt + 2 * R;
+    const int gx = x0 + 4 * tx, y = y0 + ty;
     auto issue = [&](int j) {
         const int s = j % S;
         ptx::mbar_arrive_expect_tx(&full[s], G::PLANE * 4);
@@ -510,15 +542,6 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, R + 3>::NT)
             ptx::tma_load_4d(ct + 10 * T::DT + 2 * T::PT, &fu.qp, xs, y0 + R, zp, sh, &cfull[c]);
         }
     };
-    if (tid == 0) {
-        ptx::prefetch_tmap(&tf);
-#pragma unroll
-        for (int s = 0; s < S; ++s) ptx::mbar_init(&full[s], 1);
-#pragma unroll
-        for (int c = 0; c < T::CRING; ++c) ptx::mbar_init(&cfull[c], 1);
-        ptx::fence_mbar_init();
-        abort_flag = 0;
-    }
     __syncthreads();
     if (tid == 0) {
         for (int j = 0; j < S && j < P; ++j) issue(j);
@@ -533,11 +556,11 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, R + 3>::NT)
         gys = sponge(y, geo.ny, geo.sponge_w, geo.sponge_a);
     }
 
-    float qzz[W][4], qxz[W][4], qyz[W][4];
+    f2 qzz[W][2], qxz[W][2], qyz[W][2];
 #pragma unroll
     for (int kk = 0; kk < W; ++kk)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) qzz[kk][k] = qxz[kk][k] = qyz[kk][k] = 0.f;
+        for (int h = 0; h < 2; ++h) qzz[kk][h] = qxz[kk][h] = qyz[kk][h] = zero2();
 
     const bool inside = y < geo.ny && gx < geo.nx;
     for (int j = 0; j < P; ++j) {
@@ -610,14 +633,21 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, R + 3>::NT)
             if constexpr (MODE >= 1)
                 if (zo >= 0 && zo + 2 < nzt) issue_c(zo + 2);
         }
+        float fzz[4], fxz[4], fyz[4];  // of the completed output
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            unpair(qzz[0][h], fzz[2 * h], fzz[2 * h + 1]);
+            unpair(qxz[0][h], fxz[2 * h], fxz[2 * h + 1]);
+            unpair(qyz[0][h], fyz[2 * h], fyz[2 * h + 1]);
+        }
         if (zo >= 0 && inside) {
             if constexpr (!FUSED) {
                 float l[4], h[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    l[k] = fxx[k] + fyy[k] + qzz[0][k];
-                    h[k] = tti_h1(n3[0][k], n3[1][k], n3[2][k], fxx[k], fyy[k], qzz[0][k], fxy[k], qxz[0][k],
-                                  qyz[0][k]);
+                    l[k] = fxx[k] + fyy[k] + fzz[k];
+                    h[k] = tti_h1(n3[0][k], n3[1][k], n3[2][k], fxx[k], fyy[k], fzz[k], fxy[k], fxz[k],
+                                  fyz[k]);
                 }
                 const int64_t o = (int64_t)sh * dn.ss + (int64_t)(zb + zo) * dn.sz + (int64_t)y * dn.sy + gx;
                 if (vec) {
@@ -639,9 +669,9 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, R + 3>::NT)
                 float rp4[4], rq4[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const float H1q = tti_h1(cv[7][k], cv[8][k], cv[9][k], fxx[k], fyy[k], qzz[0][k], fxy[k],
-                                             qxz[0][k], qyz[0][k]);
-                    const float H2q = fxx[k] + fyy[k] + qzz[0][k] - H1q;
+                    const float H1q = tti_h1(cv[7][k], cv[8][k], cv[9][k], fxx[k], fyy[k], fzz[k], fxy[k],
+                                             fxz[k], fyz[k]);
+                    const float H2q = fxx[k] + fyy[k] + fzz[k] - H1q;
                     const float H1p = cv[1][k], H2p = cv[0][k] - H1p;
                     const float a = cv[2][k], b = cv[3][k], c = cv[4][k], d = cv[5][k], al = cv[6][k];
                     const float inv = al != 0.f ? 1.f / al : 0.f;  // alpha > 0 inside the grid
@@ -677,13 +707,13 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, R + 3>::NT)
 #pragma unroll
         for (int kk = 0; kk < W - 1; ++kk)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                qzz[kk][k] = qzz[kk + 1][k];
-                qxz[kk][k] = qxz[kk + 1][k];
-                qyz[kk][k] = qyz[kk + 1][k];
+            for (int h = 0; h < 2; ++h) {
+                qzz[kk][h] = qzz[kk + 1][h];
+                qxz[kk][h] = qxz[kk + 1][h];
+                qyz[kk][h] = qyz[kk + 1][h];
             }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) qzz[W - 1][k] = qxz[W - 1][k] = qyz[W - 1][k] = 0.f;
+        for (int h = 0; h < 2; ++h) qzz[W - 1][h] = qxz[W - 1][h] = qyz[W - 1][h] = zero2();
     }
 }
 
@@ -777,16 +807,17 @@ cudaError_t tti_deriv_r(const WaveGeo &g, const TtiCoef &cf, const float *f, con
     Slots sl;
     cudaError_t e = kernel_slots(cache, reinterpret_cast<const void *>(kern), G::NT, T::SMEM, &sl);
     if (e != cudaSuccess) return e;
-    const int tiles_x = (g.nx + kTtiTX - 1) / kTtiTX, tiles_y = (g.ny + kTtiTY - 1) / kTtiTY;
-    const int tz = z_chunk(sl, (int64_t)tiles_x * tiles_y * g.nshots, g.nz, 2 * R, kTtiTZ, G::NT);
-    const int nzc = (g.nz + tz - 1) / tz;
-    const dim3 grid(tiles_x, tiles_y, nzc * g.nshots);
+    int64_t ctas;
+    size_t smem = T::SMEM;
+    const March march = plan_march(sl, (g.nx + kTtiTX - 1) / kTtiTX, (g.ny + kTtiTY - 1) / kTtiTY, g.nshots, g.nz,
+                                   2 * R, kTtiTZ, G::NT, &smem, &ctas);
+    if (ctas > INT32_MAX) return cudaErrorInvalidConfiguration;
     int vec = g.nx % 4 == 0 && reinterpret_cast<uintptr_t>(tilt) % 16 == 0 &&
               reinterpret_cast<uintptr_t>(lap) % 16 == 0 && reinterpret_cast<uintptr_t>(h1) % 16 == 0;
     if (MODE == 2)
         vec = g.py % 4 == 0 && g.pz % 4 == 0 && g.ss % 4 == 0 && reinterpret_cast<uintptr_t>(fu.pn) % 16 == 0 &&
               reinterpret_cast<uintptr_t>(fu.qn) % 16 == 0;
-    kern<<<grid, G::NT, T::SMEM, st>>>(tf, cf, g, tilt, dn, lap, h1, fu, tz, nzc, vec, device_error_word());
+    kern<<<(unsigned)ctas, G::NT, smem, st>>>(tf, cf, g, tilt, dn, lap, h1, fu, march, vec, device_error_word());
     return cudaGetLastError();
 }
 
@@ -851,13 +882,14 @@ cudaError_t vti_launch(const WaveGeo &g, const StarCoef &cf, int tz, const float
     Slots sl;
     cudaError_t e = kernel_slots(cache, reinterpret_cast<const void *>(kern), G::NT, V::SMEM, &sl);
     if (e != cudaSuccess) return e;
-    const int tiles_x = (g.nx + TX - 1) / TX, tiles_y = (g.ny + TY - 1) / TY;
-    tz = z_chunk(sl, (int64_t)tiles_x * tiles_y * g.nshots, g.nz, 2 * R, tz, G::NT);
-    const int nzc = (g.nz + tz - 1) / tz;
-    const dim3 grid(tiles_x, tiles_y, nzc * g.nshots);
+    int64_t ctas;
+    size_t smem = V::SMEM;
+    const March march = plan_march(sl, (g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, g.nshots, g.nz, 2 * R, tz, G::NT,
+                                   &smem, &ctas);
+    if (ctas > INT32_MAX) return cudaErrorInvalidConfiguration;
     const int vec = (R % 4 == 0) && g.py % 4 == 0 && g.pz % 4 == 0 && g.ss % 4 == 0 &&
                     reinterpret_cast<uintptr_t>(hnext) % 16 == 0 && reinterpret_cast<uintptr_t>(vnext) % 16 == 0;
-    kern<<<grid, G::NT, V::SMEM, st>>>(tm, cf, g, hnext, vnext, amp, rec, tz, nzc, vec, device_error_word());
+    kern<<<(unsigned)ctas, G::NT, smem, st>>>(tm, cf, g, hnext, vnext, amp, rec, march, vec, device_error_word());
     return cudaGetLastError();
 }
 
@@ -899,7 +931,7 @@ cudaError_t launch_vti_step(const WaveGeo &g, const float *coeffs, const float *
                             float *hnext, float *vnext, const float *src_amp, float *rec, cudaStream_t st)
 {
     StarCoef cf{};
-    for (int i = 0; i < 3 * (2 * g.r + 1); ++i) cf.c[i] = coeffs[i];
+    cf.set(coeffs, 3 * (2 * g.r + 1));
     const int v = g_vti_variant;
     switch (g.r) {
         case 1: return vti_r<1>(v, g, cf, mv, rho, hcur, vcur, hprev, vprev, hnext, vnext, src_amp, rec, st);
@@ -916,8 +948,8 @@ cudaError_t launch_tti_step(const WaveGeo &g, const float *w2, const float *w1, 
 {
     TtiCoef cf{};
     for (int i = 0; i < 2 * g.r + 1; ++i) {
-        cf.w2[i] = w2[i];
-        cf.w1[i] = w1[i];
+        cf.w2[i] = W2{w2[i], w2[i]};
+        cf.w1[i] = W2{w1[i], w1[i]};
     }
     const int64_t n = (int64_t)g.nx * g.ny * g.nz;
     TtiDense dn{g.nx, (int64_t)g.nx * g.ny, n};

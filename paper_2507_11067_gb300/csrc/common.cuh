@@ -19,8 +19,18 @@ constexpr int kMaxStar = 3 * (2 * kMaxR + 1);
 constexpr int kMaxBox = (2 * kMaxR + 1) * (2 * kMaxR + 1) * (2 * kMaxR + 1);
 
 // Coefficients travel as kernel parameters (constant bank), so every FMA
-// reads its weight as a uniform constant operand.
-struct StarCoef { float c[kMaxStar]; };
+// reads its weight as a uniform constant operand.  The star updates work on
+// pairs of points (tile.cuh), so their weights come as pairs (c, c).
+struct W2 {
+    float lo, hi;
+};
+struct StarCoef {
+    W2 c[kMaxStar];
+    void set(const float *w, int n)
+    {
+        for (int i = 0; i < n; ++i) c[i] = W2{w[i], w[i]};
+    }
+};
 struct BoxCoef { float c[kMaxBox]; };
 
 // Device error word bits (read by mms_check_device).
@@ -83,23 +93,64 @@ bool encode_tmap_3d(CUtensorMap *map, const float *base, int64_t X, int64_t Y, i
 bool encode_tmap_4d(CUtensorMap *map, const float *base, int64_t X, int64_t Y, int64_t Z,
                     int64_t W, int64_t py, int64_t pz, int64_t pw, int bx, int by, int bz);
 
+// Shared memory of an SM, what the system keeps of it per CTA, and the most
+// a CTA may ask for (sm_103).
+constexpr size_t kSmemPerSm = 228 * 1024, kSmemReserved = 1024, kSmemPerCta = 227 * 1024;
+
 // What one kernel instance can keep resident on a device, asked once per
-// device (with its dynamic shared-memory limit set to `limit`, by default
-// `smem`; launches of one kernel with several sizes pass the largest): the SM
-// count and the CTAs of `threads` threads and `smem` bytes one SM holds.  One
-// static cache per kernel instance and size; concurrent first calls compute
-// the same values.
+// device (with its dynamic shared-memory limit raised to the most there is):
+// the SM count and the CTAs of `threads` threads and `smem` bytes one SM
+// holds.  One static cache per kernel instance and size; concurrent first
+// calls compute the same values.
 struct SlotCache {
     static constexpr int kDevs = 64;
     std::atomic<uint32_t> v[kDevs];  // SMs << 8 | CTAs per SM, 0 = not asked yet
 };
 struct Slots { int sms = 0, per_sm = 0; };
-cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t smem, Slots *out, size_t limit = 0);
+cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t smem, Slots *out);
 
 // Planes per z chunk of a kernel whose CTAs each march one chunk of one of
-// `cols` columns (reading `halo` extra planes), given the kernel's tuned
-// chunk `tz`.
+// `cols` columns (reading `halo` extra planes), given the kernel's tuned chunk
+// `tz`.  A march takes (planes + halo) steps, so a launch that leaves the
+// device half empty takes about (t + halo) x the busiest SM's CTAs; the chunk
+// t is the one that makes this least among those that give an SM 1, 2, ...
+// CTAs.  A grid whose tuned chunks keep every SM busy keeps them: it is bound
+// by memory, and finer chunks only read more halo planes (box r = 1, 512^3:
+// 172 us, 196 us in finer ones).
 int z_chunk(const Slots &sl, int64_t cols, int64_t nz, int halo, int tz, int threads);
+
+// How a kernel's CTAs divide the columns they march along z: CTA b marches
+// chunk zc (tz planes) of one x, y tile of one shot, the shots fastest, then
+// x, y, chunks -- the shots of a tile read the same medium, so next to each
+// other they read it from L2 (acoustic step, 8 x 512^3, shots slowest: 3.00
+// ms, fastest: 2.83 ms).
+struct March {
+    int tiles_x, tiles_y, nshots, tz;
+};
+// The march of a launch of tuned chunk `tz`, and its grid size.  *smem, the
+// kernel's dynamic shared memory, is raised where the grid is one wave of
+// fewer CTAs than an SM holds, to what lets no SM take more than its share:
+// the scheduler doubles up on some SMs while others run one CTA (232 CTAs of
+// the VTI step on 152 SMs: one to three per SM).
+March plan_march(const Slots &sl, int64_t tiles_x, int64_t tiles_y, int nshots, int64_t nz, int halo, int tz,
+                 int threads, size_t *smem, int64_t *ctas);
+
+// The tile, shot and z chunk of this CTA.
+struct Leg {
+    int tx, ty, shot, zc;
+};
+__device__ __forceinline__ Leg leg_of(const March &m)
+{
+    unsigned b = blockIdx.x;
+    Leg g;
+    g.shot = b % m.nshots;
+    b /= m.nshots;
+    g.tx = b % m.tiles_x;
+    b /= m.tiles_x;
+    g.ty = b % m.tiles_y;
+    g.zc = b / m.tiles_y;
+    return g;
+}
 
 }  // namespace mms
 

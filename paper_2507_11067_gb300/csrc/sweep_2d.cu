@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
             ptx::mbar_arrive_expect_tx(&full[sp], G::PLANE * sizeof(float));
             ptx::tma_load_3d(stages + sp * G::STAGE, &tmap, x0, (t0 + j - 1 + S) * TY, z, &full[sp]);
         }
-        float o[PY][4];
+        f2 o[PY][2];
         if constexpr (BOX)
             box2d_tile<R, PY, G::BX, G::NV>(stages + s * G::STAGE, cf, o, tx, ry0);
         else
@@ -68,12 +68,15 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
             const int y = (t0 + j) * TY + ry0 + i;
             if (y >= ny || gx >= nx) continue;
             float *op = out + (int64_t)z * opz + (int64_t)y * opy + gx;
+            float v[4];
+            unpair(o[i][0], v[0], v[1]);
+            unpair(o[i][1], v[2], v[3]);
             if (vec_store && gx + 3 < nx) {
-                *reinterpret_cast<float4 *>(op) = make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
+                *reinterpret_cast<float4 *>(op) = make_float4(v[0], v[1], v[2], v[3]);
             } else {
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    if (gx + k < nx) op[k] = o[i][k];
+                    if (gx + k < nx) op[k] = v[k];
             }
         }
     }
@@ -149,7 +152,7 @@ cudaError_t launch_plane_cc(const Sweep &s, const CUtensorMap &tmap, int v)
         }
     }
     StarCoef cf{};
-    for (int i = 0; i < 2 * w; ++i) cf.c[i] = s.coeffs[i];
+    cf.set(s.coeffs, 2 * w);
     switch (s.r) {
         case 1: return dispatch_plane<1, false>(s, tmap, cf, v);
         case 2: return dispatch_plane<2, false>(s, tmap, cf, v);

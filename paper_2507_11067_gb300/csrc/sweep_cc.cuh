@@ -42,7 +42,7 @@ cudaError_t launch_box_cc_high(const Sweep &s, const CUtensorMap &tmap, const Bo
 template <int R, int TX, int TY, int PY, int S, bool BOX, int ROT, bool ONEW, typename Coef>
 __device__ __forceinline__ bool plane_step(int j, int P, const CUtensorMap &tmap, const Coef &cf,
                                            float *planes, uint64_t *full, int &abort_flag,
-                                           float (&acc)[2 * R + 1][PY][4], float *out, int nx, int ny,
+                                           f2 (&acc)[2 * R + 1][PY][2], float *out, int nx, int ny,
                                            int64_t opy, int64_t opz, int x0, int y0, int zb, int tx,
                                            int ry0, int gx, int vec_store, unsigned *err)
 {
@@ -50,8 +50,9 @@ __device__ __forceinline__ bool plane_step(int j, int P, const CUtensorMap &tmap
     constexpr int W = G::W;
     constexpr int Q = ROT < 0 ? 0 : ROT;  // physical slot of the oldest partial sum
     const int s = j % S;
+    const uint32_t phase = (uint32_t)(j / S) & 1u;
     if constexpr (ONEW) {
-        if (threadIdx.x == 0 && !ptx::mbar_wait_bounded(&full[s], (uint32_t)(j / S) & 1u, err)) abort_flag = 1;
+        if (threadIdx.x == 0 && !ptx::mbar_wait_bounded(&full[s], phase, err)) abort_flag = 1;
         __syncthreads();  // stage s is full for all, and every thread is done with plane j-1
         if (abort_flag) return false;
         if (threadIdx.x == 0 && j >= 1 && j - 1 + S < P) {
@@ -62,19 +63,15 @@ __device__ __forceinline__ bool plane_step(int j, int P, const CUtensorMap &tmap
         const float *pl = planes + s * G::STAGE;
         if constexpr (BOX)
             box_plane<R, PY, G::BX, G::NV, Q>(pl, cf, acc, tx, ry0);
-        else {
-            float ctr[PY][4];
-            star_plane<R, PY, G::BX, G::NV, Q>(pl, cf, acc, ctr, tx, ry0);
-        }
+        else
+            star_plane<R, PY, G::BX, G::NV, Q>(pl, cf, acc, tx, ry0);
     } else {
-        if (ptx::mbar_wait_bounded(&full[s], (uint32_t)(j / S) & 1u, err)) {
+        if (ptx::mbar_wait_bounded(&full[s], phase, err)) {
             const float *pl = planes + s * G::STAGE;
             if constexpr (BOX)
                 box_plane<R, PY, G::BX, G::NV, Q>(pl, cf, acc, tx, ry0);
-            else {
-                float ctr[PY][4];
-                star_plane<R, PY, G::BX, G::NV, Q>(pl, cf, acc, ctr, tx, ry0);
-            }
+            else
+                star_plane<R, PY, G::BX, G::NV, Q>(pl, cf, acc, tx, ry0);
         } else {
             abort_flag = 1;
         }
@@ -93,13 +90,15 @@ __device__ __forceinline__ bool plane_step(int j, int P, const CUtensorMap &tmap
             const int y = y0 + ry0 + i;
             if (y < ny && gx < nx) {
                 float *o = out + zoff + (int64_t)y * opy + gx;
+                float v[4];
+                unpair(acc[Q][i][0], v[0], v[1]);
+                unpair(acc[Q][i][1], v[2], v[3]);
                 if (vec_store && gx + 3 < nx) {
-                    *reinterpret_cast<float4 *>(o) =
-                        make_float4(acc[Q][i][0], acc[Q][i][1], acc[Q][i][2], acc[Q][i][3]);
+                    *reinterpret_cast<float4 *>(o) = make_float4(v[0], v[1], v[2], v[3]);
                 } else {
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        if (gx + k < nx) o[k] = acc[Q][i][k];
+                        if (gx + k < nx) o[k] = v[k];
                 }
             }
         }
@@ -110,14 +109,14 @@ __device__ __forceinline__ bool plane_step(int j, int P, const CUtensorMap &tmap
 #pragma unroll
             for (int i = 0; i < PY; ++i)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[kk][i][k] = acc[kk + 1][i][k];
+                for (int h = 0; h < 2; ++h) acc[kk][i][h] = acc[kk + 1][i][h];
     }
     // the freed slot becomes the newest output plane's
     constexpr int FREE = ROT < 0 ? W - 1 : Q;
 #pragma unroll
     for (int i = 0; i < PY; ++i)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[FREE][i][k] = 0.f;
+        for (int h = 0; h < 2; ++h) acc[FREE][i][h] = zero2();
     return true;
 }
 
@@ -128,7 +127,7 @@ template <int R, int TX, int TY, int PY, int S, bool BOX, bool ONEW, typename Co
 __device__ __forceinline__ bool rotated_block(std::integer_sequence<int, U...>, int j0, int P,
                                               const CUtensorMap &tmap, const Coef &cf, float *planes,
                                               uint64_t *full, int &abort_flag,
-                                              float (&acc)[2 * R + 1][PY][4], float *out, int nx, int ny,
+                                              f2 (&acc)[2 * R + 1][PY][2], float *out, int nx, int ny,
                                               int64_t opy, int64_t opz, int x0, int y0, int zb, int tx,
                                               int ry0, int gx, int vec_store, unsigned *err)
 {
@@ -145,7 +144,7 @@ template <int R, int TX, int TY, int PY, int S, bool BOX, bool ROTQ, bool ONEW, 
 __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
     sweep_cc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ Coef cf,
                     float *__restrict__ out, int nx, int ny, int nz, int64_t opy, int64_t opz,
-                    int tz, int vec_store, unsigned *err)
+                    const __grid_constant__ March march, int vec_store, unsigned *err)
 {
     using G = Geom<R, TX, TY, PY, S>;
     constexpr int W = G::W;
@@ -157,11 +156,7 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
 
     const int tid = threadIdx.x;
     const int tx = tid % G::NTX, ty = tid / G::NTX;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, zb = blockIdx.z * tz;
-    const int nzt = min(tz, nz - zb);
-    const int P = nzt + 2 * R;  // padded planes this CTA consumes
     const int ry0 = ty * PY;
-    const int gx = x0 + 4 * tx;
 
     if (tid == 0) {
         ptx::prefetch_tmap(&tmap);
@@ -170,21 +165,24 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
         ptx::fence_mbar_init();
         abort_flag = 0;
     }
+    const Leg leg = leg_of(march);
+    const int x0 = leg.tx * TX, y0 = leg.ty * TY, zb = leg.zc * march.tz;
+    const int P = min(march.tz, nz - zb) + 2 * R;  // padded planes this CTA consumes
+    const int gx = x0 + 4 * tx;
     __syncthreads();
     if (tid == 0) {
         for (int j = 0; j < S && j < P; ++j) {
-            ptx::mbar_arrive_expect_tx(&full[j], G::PLANE * sizeof(float));
-            ptx::tma_load_3d(planes + j * G::STAGE, &tmap, x0, y0, zb + j, &full[j]);
+            const int s = j;
+            ptx::mbar_arrive_expect_tx(&full[s], G::PLANE * sizeof(float));
+            ptx::tma_load_3d(planes + s * G::STAGE, &tmap, x0, y0, zb + j, &full[s]);
         }
     }
 
-    float acc[W][PY][4];
+    f2 acc[W][PY][2];
 #pragma unroll
     for (int kk = 0; kk < W; ++kk)
 #pragma unroll
-        for (int i = 0; i < PY; ++i)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[kk][i][k] = 0.f;
+        for (int i = 0; i < PY; ++i) acc[kk][i][0] = acc[kk][i][1] = zero2();
 
     // The box rotates only for R <= 2: above that its 2R+1 unrolled copies
     // of a (2R+1)^3-term plane update cost more than the moves they save.
@@ -193,16 +191,15 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
         // 2R+1 planes per iteration, so every queue slot index is a constant
         // and no partial sum is moved between registers
         for (int j0 = 0; j0 < P; j0 += W)
-            if (!rotated_block<R, TX, TY, PY, S, BOX, ONEW, Coef>(std::make_integer_sequence<int, W>{}, j0, P,
-                                                            tmap, cf, planes, full, abort_flag, acc, out,
-                                                            nx, ny, opy, opz, x0, y0, zb, tx, ry0, gx,
-                                                            vec_store, err))
+            if (!rotated_block<R, TX, TY, PY, S, BOX, ONEW, Coef>(
+                    std::make_integer_sequence<int, W>{}, j0, P, tmap, cf, planes, full, abort_flag, acc,
+                    out, nx, ny, opy, opz, x0, y0, zb, tx, ry0, gx, vec_store, err))
                 return;
     } else {
         for (int j = 0; j < P; ++j)
-            if (!plane_step<R, TX, TY, PY, S, BOX, -1, ONEW>(j, P, tmap, cf, planes, full, abort_flag, acc, out,
-                                                       nx, ny, opy, opz, x0, y0, zb, tx, ry0, gx,
-                                                       vec_store, err))
+            if (!plane_step<R, TX, TY, PY, S, BOX, -1, ONEW>(j, P, tmap, cf, planes, full, abort_flag, acc,
+                                                             out, nx, ny, opy, opz, x0, y0, zb, tx, ry0, gx,
+                                                             vec_store, err))
                 return;
     }
 }
@@ -217,15 +214,16 @@ cudaError_t launch_tiled(const Sweep &sw, const CUtensorMap &tmap, const Coef &c
     cudaError_t e = kernel_slots(cache, reinterpret_cast<const void *>(kern), G::NT, G::SMEM, &sl);
     if (e != cudaSuccess) return e;
     const int64_t tiles_x = (sw.nx + TX - 1) / TX, tiles_y = (sw.ny + TY - 1) / TY;
-    tz = z_chunk(sl, tiles_x * tiles_y, sw.nz, 2 * R, tz, G::NT);
-    const dim3 grid((unsigned)tiles_x, (unsigned)tiles_y, (unsigned)((sw.nz + tz - 1) / tz));
+    int64_t ctas;
+    size_t smem = G::SMEM;
+    const March march = plan_march(sl, tiles_x, tiles_y, 1, sw.nz, 2 * R, tz, G::NT, &smem, &ctas);
+    if (ctas > INT32_MAX) return cudaErrorInvalidConfiguration;
     const int vec = ((sw.opy % 4) == 0 && (sw.opz % 4) == 0 &&
                      (reinterpret_cast<uintptr_t>(sw.out) % 16) == 0)
                         ? 1
                         : 0;
-    kern<<<grid, G::NT, G::SMEM, sw.stream>>>(tmap, cf, sw.out, (int)sw.nx, (int)sw.ny,
-                                               (int)sw.nz, sw.opy, sw.opz, tz, vec,
-                                               device_error_word());
+    kern<<<(unsigned)ctas, G::NT, smem, sw.stream>>>(tmap, cf, sw.out, (int)sw.nx, (int)sw.ny, (int)sw.nz, sw.opy,
+                                                        sw.opz, march, vec, device_error_word());
     return cudaGetLastError();
 }
 

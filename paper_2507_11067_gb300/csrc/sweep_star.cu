@@ -42,7 +42,7 @@ cudaError_t launch_star_cc(const Sweep &s, const CUtensorMap &tmap, int v)
 {
     StarCoef cf{};
     const int w = 2 * s.r + 1;
-    for (int i = 0; i < 3 * w; ++i) cf.c[i] = s.coeffs[i];
+    cf.set(s.coeffs, 3 * w);
     switch (s.r) {
         case 1: return dispatch_star<1>(s, tmap, cf, v);
         case 2: return dispatch_star<2>(s, tmap, cf, v);

@@ -64,39 +64,103 @@ __device__ __forceinline__ void load_center(const float *p, float (&v)[4])
     }
 }
 
+// ---------------------------------------------------------------- pairs
+// Two neighbouring points in one 64-bit register pair.  fma.rn.f32x2 is the
+// same two IEEE FMAs in one instruction: the FP32 pipe does no more of them
+// per clock (73 against 76 TFLOP/s measured), but a plane update issues half
+// as many instructions, and issue is what binds these kernels (64 to 91 % of
+// the cycles against 36 % for the pipe).
+using f2 = float2;
+
+__device__ __forceinline__ f2 pair(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ f2 pair(const W2 &w) { return make_float2(w.lo, w.hi); }
+__device__ __forceinline__ f2 zero2() { return make_float2(0.f, 0.f); }
+__device__ __forceinline__ void unpair(const f2 &v, float &a, float &b)
+{
+    a = v.x;
+    b = v.y;
+}
+__device__ __forceinline__ f2 fma2(const f2 &a, const f2 &b, const f2 &c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ f2 mul2(const f2 &a, const f2 &b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ f2 add2(const f2 &a, const f2 &b) { return __fadd2_rn(a, b); }
+
+// Whether a star update of radius R works on pairs: radius 3 and 4 are bound
+// by issue (1024^3: r = 4 1.62 -> 1.39 ms, r = 3 1.40 -> 1.37 ms, HBM at 91
+// %); at r = 1, 2 HBM binds already and pairs only cost registers (r = 2:
+// 1.29 -> 1.55 ms).  The boxes are bound by the FMA pipe, which pairs do not
+// relieve (r = 1, 512^3: 171 -> 188 us; 2D box r = 3: 117 -> 119 us).
+template <int R>
+constexpr bool kPairs = R >= 3;
+
+// acc += w * v over a pair of points; point by point (WHOLE false) where v's
+// halves do not share an aligned register pair: the moves that would pair them
+// cost as much as the FMA they save, and take the FMA pipe as well.
+template <bool WHOLE>
+__device__ __forceinline__ void fma_pair(const W2 &w, const f2 &v, f2 &acc)
+{
+    if constexpr (WHOLE) {
+        acc = fma2(pair(w), v, acc);
+    } else {
+        acc.x = fmaf(w.lo, v.x, acc.x);
+        acc.y = fmaf(w.lo, v.y, acc.y);
+    }
+}
+
+// acc (points 0..3 as two pairs) += sum_d w[d + R] * row[k + R + d], d
+// ascending, over the 4 points k of a window row.  A tap whose columns start
+// on an even register pairs with its neighbour.
+template <int R>
+__device__ __forceinline__ void line_x(const W2 *w, const float *row, f2 (&acc)[2])
+{
+#pragma unroll
+    for (int d = -R; d <= R; ++d)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const f2 v = pair(row[2 * h + R + d], row[2 * h + R + d + 1]);
+            if (kPairs<R> && (R + d) % 2 == 0) fma_pair<true>(w[d + R], v, acc[h]);
+            else fma_pair<false>(w[d + R], v, acc[h]);
+        }
+}
+
+// The centre values (columns R..R+3) of a staged row, as two pairs.
+template <int R>
+__device__ __forceinline__ void load_center2(const float *p, f2 (&v)[2])
+{
+    float c[4];
+    load_center<R>(p, c);
+    v[0] = pair(c[0], c[1]);
+    v[1] = pair(c[2], c[3]);
+}
+
 // Queue slots: logical slot kk (output plane j - 2R + kk for input plane j)
 // lives in acc[(kk + ROT) % (2R+1)]; ROT = 0 for a queue that is shifted
-// after every plane, a compile-time rotation for one that is not.
+// after every plane, a compile-time rotation for one that is not.  A point's
+// four x neighbours are two pairs.
 //
 // Star: plane j adds c_z[R-kk] * centre to the output plane at queue slot kk
-// and its in-plane x/y part to slot R (the plane it centres); the centre
-// values of the thread's points are returned in ctr.
+// and its in-plane x/y part to slot R (the plane it centres).
 template <int R, int PY, int BX, int NV, int ROT = 0>
-__device__ __forceinline__ void star_plane(const float *pl, const StarCoef &cf,
-                                           float (&acc)[2 * R + 1][PY][4], float (&ctr)[PY][4],
-                                           int tx, int ry0)
+__device__ __forceinline__ void star_plane(const float *pl, const StarCoef &cf, f2 (&acc)[2 * R + 1][PY][2], int tx,
+                                           int ry0)
 {
     constexpr int W = 2 * R + 1;
-    float cen[PY + 2 * R][4];
+    f2 cen[PY + 2 * R][2];
 #pragma unroll
-    for (int rr = 0; rr < PY + 2 * R; ++rr) load_center<R>(pl + (ry0 + rr) * BX + 4 * tx, cen[rr]);
+    for (int rr = 0; rr < PY + 2 * R; ++rr) load_center2<R>(pl + (ry0 + rr) * BX + 4 * tx, cen[rr]);
 #pragma unroll
     for (int i = 0; i < PY; ++i) {
         float win[4 * NV];
         load_row<NV>(pl + (ry0 + R + i) * BX + 4 * tx, win);
+        f2 xy[2] = {zero2(), zero2()};
+        line_x<R>(cf.c, win, xy);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float c0 = cen[i + R][k];
-            ctr[i][k] = c0;
-            float xy = 0.f;
+        for (int h = 0; h < 2; ++h) {
 #pragma unroll
-            for (int d = -R; d <= R; ++d) xy = fmaf(cf.c[0 * W + d + R], win[k + R + d], xy);
-#pragma unroll
-            for (int d = -R; d <= R; ++d) xy = fmaf(cf.c[1 * W + d + R], cen[i + R + d][k], xy);
-            acc[(R + ROT) % W][i][k] += xy;
+            for (int d = -R; d <= R; ++d) fma_pair<kPairs<R> && R % 2 == 0>(cf.c[1 * W + d + R], cen[i + R + d][h], xy[h]);
+            acc[(R + ROT) % W][i][h] = add2(acc[(R + ROT) % W][i][h], xy[h]);
 #pragma unroll
             for (int kk = 0; kk < W; ++kk)
-                acc[(kk + ROT) % W][i][k] = fmaf(cf.c[2 * W + 2 * R - kk], c0, acc[(kk + ROT) % W][i][k]);
+                fma_pair<kPairs<R> && R % 2 == 0>(cf.c[2 * W + 2 * R - kk], cen[i + R][h], acc[(kk + ROT) % W][i][h]);
         }
     }
 }
@@ -104,8 +168,8 @@ __device__ __forceinline__ void star_plane(const float *pl, const StarCoef &cf,
 // Box: window row rr of the plane feeds output row i with dy = rr - R - i;
 // slot kk (output plane z_o) takes the weights of dz = R - kk.
 template <int R, int PY, int BX, int NV, int ROT = 0>
-__device__ __forceinline__ void box_plane(const float *pl, const BoxCoef &cf,
-                                          float (&acc)[2 * R + 1][PY][4], int tx, int ry0)
+__device__ __forceinline__ void box_plane(const float *pl, const BoxCoef &cf, f2 (&acc)[2 * R + 1][PY][2], int tx,
+                                          int ry0)
 {
     constexpr int W = 2 * R + 1;
 #pragma unroll
@@ -121,11 +185,12 @@ __device__ __forceinline__ void box_plane(const float *pl, const BoxCoef &cf,
                 const int dz = R - kk;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    float a = acc[(kk + ROT) % W][i][k];
+                    f2 &q = acc[(kk + ROT) % W][i][k / 2];
+                    float a = k % 2 ? q.y : q.x;
 #pragma unroll
                     for (int dx = -R; dx <= R; ++dx)
                         a = fmaf(cf.c[((dz + R) * W + dy + R) * W + dx + R], row[k + R + dx], a);
-                    acc[(kk + ROT) % W][i][k] = a;
+                    (k % 2 ? q.y : q.x) = a;
                 }
             }
         }
@@ -135,39 +200,33 @@ __device__ __forceinline__ void box_plane(const float *pl, const BoxCoef &cf,
 // Planar star (Table I's 2D kernels): the thread's 4 x PY outputs of a staged
 // tile, x line (weights c[0..2R]) plus y line (weights c[2R+1..4R+1]).
 template <int R, int PY, int BX, int NV>
-__device__ __forceinline__ void star2d_tile(const float *pl, const StarCoef &cf, float (&o)[PY][4], int tx,
-                                            int ry0)
+__device__ __forceinline__ void star2d_tile(const float *pl, const StarCoef &cf, f2 (&o)[PY][2], int tx, int ry0)
 {
     constexpr int W = 2 * R + 1;
-    float cen[PY + 2 * R][4];
+    f2 cen[PY + 2 * R][2];
 #pragma unroll
-    for (int rr = 0; rr < PY + 2 * R; ++rr) load_center<R>(pl + (ry0 + rr) * BX + 4 * tx, cen[rr]);
+    for (int rr = 0; rr < PY + 2 * R; ++rr) load_center2<R>(pl + (ry0 + rr) * BX + 4 * tx, cen[rr]);
 #pragma unroll
     for (int i = 0; i < PY; ++i) {
         float win[4 * NV];
         load_row<NV>(pl + (ry0 + R + i) * BX + 4 * tx, win);
+        o[i][0] = o[i][1] = zero2();
+        line_x<R>(cf.c, win, o[i]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            float acc = 0.f;
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int d = -R; d <= R; ++d) acc = fmaf(cf.c[d + R], win[k + R + d], acc);
-#pragma unroll
-            for (int d = -R; d <= R; ++d) acc = fmaf(cf.c[W + d + R], cen[i + R + d][k], acc);
-            o[i][k] = acc;
-        }
+            for (int d = -R; d <= R; ++d) fma_pair<kPairs<R> && R % 2 == 0>(cf.c[W + d + R], cen[i + R + d][h], o[i][h]);
     }
 }
 
 // Planar box: window row rr of the tile feeds output row i with dy = rr - R - i.
 template <int R, int PY, int BX, int NV>
-__device__ __forceinline__ void box2d_tile(const float *pl, const BoxCoef &cf, float (&o)[PY][4], int tx,
-                                           int ry0)
+__device__ __forceinline__ void box2d_tile(const float *pl, const BoxCoef &cf, f2 (&o)[PY][2], int tx, int ry0)
 {
     constexpr int W = 2 * R + 1;
 #pragma unroll
     for (int i = 0; i < PY; ++i)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o[i][k] = 0.f;
+        for (int h = 0; h < 2; ++h) o[i][h] = zero2();
 #pragma unroll
     for (int rr = 0; rr < PY + 2 * R; ++rr) {
         float row[4 * NV];
@@ -179,8 +238,10 @@ __device__ __forceinline__ void box2d_tile(const float *pl, const BoxCoef &cf, f
 #pragma unroll
             for (int k = 0; k < 4; ++k)
 #pragma unroll
-                for (int dx = -R; dx <= R; ++dx)
-                    o[i][k] = fmaf(cf.c[(dy + R) * W + dx + R], row[k + R + dx], o[i][k]);
+                for (int dx = -R; dx <= R; ++dx) {
+                    float &q = k % 2 ? o[i][k / 2].y : o[i][k / 2].x;
+                    q = fmaf(cf.c[(dy + R) * W + dx + R], row[k + R + dx], q);
+                }
         }
     }
 }

@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
                     const __grid_constant__ CUtensorMap tlap, const __grid_constant__ StarCoef cf,
                     const __grid_constant__ WaveGeo geo, float *__restrict__ pnext,
                     const float *__restrict__ amp, float *__restrict__ rec, float *__restrict__ lapout,
-                    const __grid_constant__ AdjArgs adj, int tz, int nzc, int vec, unsigned *err)
+                    const __grid_constant__ AdjArgs adj, const __grid_constant__ March march, int vec, unsigned *err)
 {
     constexpr bool LAPOUT = MODE == K_FWD_LAP;
     constexpr bool ADJ = MODE == K_ADJ_SCALED;
@@ -194,19 +194,7 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
     launch_dependents();
     const int tid = threadIdx.x;
     const int tx = tid % G::NTX, ty = tid / G::NTX;
-    // The adjoint's shots of one z chunk are adjacent in launch order, so
-    // that they run together and their FP64 gradient rows meet in L2 (its
-    // z chunks can span several waves); the forward forms keep a shot's
-    // chunks adjacent (measured faster for them: 8 x 512^3, 2.97 against
-    // 3.25 ms per step).
-    const int sh = ADJ ? blockIdx.z % geo.nshots : blockIdx.z / nzc;
-    const int zc = ADJ ? blockIdx.z / geo.nshots : blockIdx.z % nzc;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, zb = zc * tz;
-    const int nzt = min(tz, geo.nz - zb);
-    const int P = nzt + 2 * R;
     const int ry0 = ty * PY;
-    const int gx = x0 + 4 * tx;
-    const int sx = ADJ ? -1 : geo.src[sh][0], sy = ADJ ? -1 : geo.src[sh][1], sz = ADJ ? -1 : geo.src[sh][2];
     const bool has_grad = ADJ && adj.grad != nullptr;
     // The shots' terms go to one shared gradient: each output plane's terms
     // are gathered in shared memory and each row is added by one bulk
@@ -215,20 +203,6 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
     [[maybe_unused]] double *gbuf = reinterpret_cast<double *>(smem + F::OFF_GB);
     const int ntiles = has_grad ? 4 : 3;
 
-    auto issue = [&](int j, int s) {
-        float *st = stages + (size_t)s * F::STAGE;
-        const bool inner = j >= 2 * R;  // this plane completes output plane j - 2R
-        ptx::mbar_arrive_expect_tx(&full[s], (G::PLANE + (inner ? ntiles * F::MT : 0)) * sizeof(float));
-        ptx::tma_load_4d(st, &tcur, x0, y0, zb + j, sh, &full[s]);
-        if (inner) {
-            const int zp = zb + j - R;  // padded plane of output zo = j - 2R
-            const int xs = x0 + (R & ~3);
-            ptx::tma_load_3d(st + F::OFF_M, &tm, xs, y0 + R, zp, &full[s]);
-            ptx::tma_load_4d(st + F::OFF_P, &tprev, xs, y0 + R, zp, sh, &full[s]);
-            ptx::tma_load_4d(st + F::OFF_C, &tctr, xs, y0 + R, zp, sh, &full[s]);
-            if (has_grad) ptx::tma_load_4d(st + F::OFF_L, &tlap, xs, y0 + R, zp, sh, &full[s]);
-        }
-    };
     if (tid == 0) {
         ptx::prefetch_tmap(&tcur);
         ptx::prefetch_tmap(&tm);
@@ -242,22 +216,40 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
     }
     // the previous step's fields are complete before any is read or written
     wait_prior_grid();
+    const Leg leg = leg_of(march);
+    const int sh = leg.shot, x0 = leg.tx * TX, y0 = leg.ty * TY, zb = leg.zc * march.tz;
+    const int P = min(march.tz, geo.nz - zb) + 2 * R;
+    const int gx = x0 + 4 * tx;
+    const int sx = ADJ ? -1 : geo.src[sh][0], sy = ADJ ? -1 : geo.src[sh][1], sz = ADJ ? -1 : geo.src[sh][2];
+    auto issue = [&](int j) {
+        const int s = j % S;
+        float *st = stages + (size_t)s * F::STAGE;
+        const bool inner = j >= 2 * R;  // this plane completes output plane j - 2R
+        ptx::mbar_arrive_expect_tx(&full[s], (G::PLANE + (inner ? ntiles * F::MT : 0)) * sizeof(float));
+        ptx::tma_load_4d(st, &tcur, x0, y0, zb + j, sh, &full[s]);
+        if (inner) {
+            const int zp = zb + j - R;  // padded plane of output zo = j - 2R
+            const int xs = x0 + (R & ~3);
+            ptx::tma_load_3d(st + F::OFF_M, &tm, xs, y0 + R, zp, &full[s]);
+            ptx::tma_load_4d(st + F::OFF_P, &tprev, xs, y0 + R, zp, sh, &full[s]);
+            ptx::tma_load_4d(st + F::OFF_C, &tctr, xs, y0 + R, zp, sh, &full[s]);
+            if (has_grad) ptx::tma_load_4d(st + F::OFF_L, &tlap, xs, y0 + R, zp, sh, &full[s]);
+        }
+    };
     __syncthreads();
     if (tid == 0)
-        for (int j = 0; j < S && j < P; ++j) issue(j, j);
+        for (int j = 0; j < S && j < P; ++j) issue(j);
     float gxs[4], gys[PY];
 #pragma unroll
     for (int k = 0; k < 4; ++k) gxs[k] = sponge(gx + k, geo.nx, geo.sponge_w, geo.sponge_a);
 #pragma unroll
     for (int i = 0; i < PY; ++i) gys[i] = sponge(y0 + ry0 + i, geo.ny, geo.sponge_w, geo.sponge_a);
 
-    float acc[W][PY][4];
+    f2 acc[W][PY][2];
 #pragma unroll
     for (int kk = 0; kk < W; ++kk)
 #pragma unroll
-        for (int i = 0; i < PY; ++i)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[kk][i][k] = 0.f;
+        for (int i = 0; i < PY; ++i) acc[kk][i][0] = acc[kk][i][1] = zero2();
 
     const float samp = ADJ ? 0.f : amp[sh];
     const int64_t shot_off = (int64_t)sh * geo.ss;
@@ -268,8 +260,7 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
         float mv[PY][4], pv[PY][4], cv[PY][4];
         [[maybe_unused]] float lv[PY][4];
         if (ptx::mbar_wait_bounded(&full[s], (uint32_t)(j / S) & 1u, err)) {
-            float unused[PY][4];
-            star_plane<R, PY, G::BX, G::NV>(st, cf, acc, unused, tx, ry0);
+            star_plane<R, PY, G::BX, G::NV>(st, cf, acc, tx, ry0);
             if (zo >= 0) {
 #pragma unroll
                 for (int i = 0; i < PY; ++i) {
@@ -289,7 +280,7 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
             if constexpr (ADJ) bulk_wait_all();  // no reduction still reads this CTA's buffers
             return;
         }
-        if (tid == 0 && j + S < P) issue(j + S, s);
+        if (tid == 0 && j + S < P) issue(j + S);
         if (zo >= 0) {
             const int z = zb + zo;
             const float gzv = sponge(z, geo.nz, geo.sponge_w, geo.sponge_a);
@@ -308,13 +299,15 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
                 if (y >= geo.ny || gx >= geo.nx) continue;
                 const int64_t mp = (int64_t)(z + R) * geo.pz + (int64_t)(y + R) * geo.py + (gx + R);
                 float *pp = pnext + shot_off + mp;
-                float res[4];
+                float res[4], lap[4];
+                unpair(acc[0][i][0], lap[0], lap[1]);
+                unpair(acc[0][i][1], lap[2], lap[3]);
                 [[maybe_unused]] double gd[4] = {0.0, 0.0, 0.0, 0.0};
                 [[maybe_unused]] const bool at_rec = ADJ && adj.resid && z == geo.rec_z;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const float g = gxs[k] * gys[i] * gzv;
-                    float v = 2.f * cv[i][k] + mv[i][k] * acc[0][i][k] - g * pv[i][k];
+                    float v = 2.f * cv[i][k] + mv[i][k] * lap[k] - g * pv[i][k];
                     if constexpr (ADJ) {
                         if (at_rec && gx + k < geo.nx)
                             v += mv[i][k] * adj.resid[((int64_t)sh * geo.ny + y) * geo.nx + gx + k];
@@ -338,11 +331,11 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
                 if constexpr (LAPOUT) {  // L a^n itself, for the gradient's adjoint steps
                     float *lo = lapout + shot_off + mp;
                     if (vec && gx + 3 < geo.nx) {
-                        *reinterpret_cast<float4 *>(lo) = make_float4(acc[0][i][0], acc[0][i][1], acc[0][i][2], acc[0][i][3]);
+                        *reinterpret_cast<float4 *>(lo) = make_float4(lap[0], lap[1], lap[2], lap[3]);
                     } else {
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            if (gx + k < geo.nx) lo[k] = acc[0][i][k];
+                            if (gx + k < geo.nx) lo[k] = lap[k];
                     }
                 }
                 if (rec && z == geo.rec_z) {
@@ -407,11 +400,9 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
 #pragma unroll
             for (int i = 0; i < PY; ++i)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[kk][i][k] = acc[kk + 1][i][k];
+                for (int h = 0; h < 2; ++h) acc[kk][i][h] = acc[kk + 1][i][h];
 #pragma unroll
-        for (int i = 0; i < PY; ++i)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) acc[W - 1][i][k] = 0.f;
+        for (int i = 0; i < PY; ++i) acc[W - 1][i][0] = acc[W - 1][i][1] = zero2();
     }
     // this thread's reductions are complete before the CTA exits
     if constexpr (ADJ)
@@ -505,11 +496,11 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT, 2)
     if (tid == 0)
         for (int j = 0; j < S && j < P; ++j) issue(j, j);
 
-    float accq[W][PY][4], acca[W][PY][4];
+    f2 accq[W][PY][2], acca[W][PY][2];
 #pragma unroll
     for (int kk = 0; kk < W; ++kk)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) accq[kk][0][k] = acca[kk][0][k] = 0.f;
+        for (int h = 0; h < 2; ++h) accq[kk][0][h] = acca[kk][0][h] = zero2();
     float gxs[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) gxs[k] = gxt[4 * tx + R + k];
@@ -552,9 +543,8 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT, 2)
         if (abort_flag) return false;
         float l2v[4], l1v[4], lav[4];
         {
-            float unused[PY][4];
-            star_plane<R, PY, G::BX, G::NV, Q>(qbuf, cf, accq, unused, tx, ry0);
-            if (!LAPIN && has_a) star_plane<R, PY, G::BX, G::NV, Q>(st + 2 * A::PL, cf, acca, unused, tx, ry0);
+            star_plane<R, PY, G::BX, G::NV, Q>(qbuf, cf, accq, tx, ry0);
+            if (!LAPIN && has_a) star_plane<R, PY, G::BX, G::NV, Q>(st + 2 * A::PL, cf, acca, tx, ry0);
             if (zo >= 0) {
                 load_center<I::OFF>(st + A::OFF_L2 + ry0 * I::BXI + 4 * tx, l2v);
                 load_center<I::OFF>(st + A::OFF_L1 + ry0 * I::BXI + 4 * tx, l1v);
@@ -573,15 +563,20 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT, 2)
                 const int64_t gi = ((int64_t)z * geo.ny + y) * geo.nx + gx;
                 const bool at_rec = resid && z == geo.rec_z;
                 double gd[4] = {0.0, 0.0, 0.0, 0.0};
+                float lq[4], la[4];
+                unpair(accq[Q][0][0], lq[0], lq[1]);
+                unpair(accq[Q][0][1], lq[2], lq[3]);
+                unpair(acca[Q][0][0], la[0], la[1]);
+                unpair(acca[Q][0][1], la[2], la[3]);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     if (gx + k >= geo.nx) break;
                     const float g = gxs[k] * gys0 * gzv;
-                    float v = 2.f * g * l1v[k] + accq[Q][0][k] - g * g * l2v[k];
+                    float v = 2.f * g * l1v[k] + lq[k] - g * g * l2v[k];
                     if (at_rec) v += resid[((int64_t)sh * geo.ny + y) * geo.nx + gx + k];
                     lp[k] = v;
                     // the step's term in FP32 (its operands are FP32), accumulated in FP64
-                    if (has_a) gd[k] = widen(g * l1v[k] * (LAPIN ? lav[k] : acca[Q][0][k]));
+                    if (has_a) gd[k] = widen(g * l1v[k] * (LAPIN ? lav[k] : la[k]));
                 }
                 if (has_a) {
                     if (geo.gss == 0) {
@@ -610,12 +605,12 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT, 2)
 #pragma unroll
         for (int kk = 0; kk < W - 1; ++kk)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                accq[kk][0][k] = accq[kk + 1][0][k];
-                acca[kk][0][k] = acca[kk + 1][0][k];
+            for (int h = 0; h < 2; ++h) {
+                accq[kk][0][h] = accq[kk + 1][0][h];
+                acca[kk][0][h] = acca[kk + 1][0][h];
             }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) accq[W - 1][0][k] = acca[W - 1][0][k] = 0.f;
+        for (int h = 0; h < 2; ++h) accq[W - 1][0][h] = acca[W - 1][0][h] = zero2();
         return true;
     };
     for (int j = 0; j < P; ++j)
@@ -719,34 +714,35 @@ cudaError_t fwd_r(const WaveGeo &g, const StarCoef &cf, const float *m, const fl
     using FA = FwdGeom<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_ADJ_SCALED>;
     // the adjoint's gradient buffers only where its bulk reductions run
     const bool gbulk = adj && adj->grad && g.gss == 0 && adj->gbulk;
-    const size_t smem = mode == K_ADJ_SCALED ? FA::SMEM - (gbulk ? 0 : FA::GB_BYTES)
+    size_t smem = mode == K_ADJ_SCALED ? FA::SMEM - (gbulk ? 0 : FA::GB_BYTES)
                         : mode == K_FWD_LAP  ? FwdGeom<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_FWD_LAP>::SMEM
                                              : FwdGeom<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_FWD>::SMEM;
     static SlotCache caches[4];  // per form (the adjoint without and with its gradient buffers)
     Slots sl;
-    cudaError_t e = kernel_slots(caches[mode + (gbulk ? 1 : 0)], reinterpret_cast<const void *>(kern), G::NT, smem, &sl,
-                                 mode == K_ADJ_SCALED ? FA::SMEM : smem);
+    cudaError_t e = kernel_slots(caches[mode + (gbulk ? 1 : 0)], reinterpret_cast<const void *>(kern), G::NT, smem, &sl);
     if (e != cudaSuccess) return e;
     const int tiles_x = (g.nx + kFwdTX - 1) / kFwdTX, tiles_y = (g.ny + kFwdTY - 1) / kFwdTY;
-    const int64_t cols = (int64_t)tiles_x * tiles_y * g.nshots, slots = (int64_t)sl.sms * sl.per_sm;
-    int tz = z_chunk(sl, cols, g.nz, 2 * R, kFwdTZ, G::NT);
-    // The adjoint step on a grid whose CTAs fill most of one wave splits z
-    // finer, into about three waves, so that the SMs left with one CTA do not
-    // idle while the others finish two (2 x 256^3: 219 -> 207 us per step; the
-    // forward forms gained nothing).
-    if (mode == K_ADJ_SCALED && 2 * cols * ((g.nz + kFwdTZ - 1) / kFwdTZ) > slots &&
-        cols * ((g.nz + kFwdTZ - 1) / kFwdTZ) <= slots) {
-        const int k = (int)((3 * slots + cols / 2) / cols);  // chunks per column for about three waves
-        tz = k > 0 ? (g.nz + k - 1) / k : tz;
-        if (tz < 2 * R) tz = 2 * R;
+    int tz = kFwdTZ;
+    if (mode == K_ADJ_SCALED) {
+        // The adjoint step on a grid whose tuned chunks fill at most one wave
+        // splits z finer, into about three waves, so that the SMs left with
+        // one CTA do not idle while the others finish two (2 x 256^3: 219 ->
+        // 207 us per step; the forward forms gained nothing).
+        const int64_t cols = (int64_t)tiles_x * tiles_y * g.nshots, slots = (int64_t)sl.sms * sl.per_sm;
+        if (cols * ((g.nz + tz - 1) / tz) <= slots) {
+            const int64_t k = (3 * slots + cols / 2) / cols;  // chunks per column for about three waves
+            tz = (int)((g.nz + k - 1) / k);
+            if (tz < 2 * R) tz = 2 * R;
+        }
     }
-    const int nzc = (g.nz + tz - 1) / tz;
-    const dim3 grid(tiles_x, tiles_y, nzc * g.nshots);
+    int64_t ctas;
+    const March march = plan_march(sl, tiles_x, tiles_y, g.nshots, g.nz, 2 * R, tz, G::NT, &smem, &ctas);
+    if (ctas > INT32_MAX) return cudaErrorInvalidConfiguration;
     const int vec = (R % 4 == 0) && g.py % 4 == 0 && g.pz % 4 == 0 && g.ss % 4 == 0 &&
                     reinterpret_cast<uintptr_t>(p_next) % 16 == 0 && reinterpret_cast<uintptr_t>(lapout) % 16 == 0;
     const AdjArgs aa = adj ? *adj : AdjArgs{nullptr, nullptr, 0, 0};
-    return launch_overlapped(kern, grid, dim3(G::NT), smem, st, mcur, mm, mprev, mctr, mlap, cf, g, p_next, amp, rec,
-                             lapout, aa, tz, nzc, vec, device_error_word());
+    return launch_overlapped(kern, dim3((unsigned)ctas), dim3(G::NT), smem, st, mcur, mm, mprev, mctr, mlap, cf, g,
+                             p_next, amp, rec, lapout, aa, march, vec, device_error_word());
 }
 
 template <int R, bool LAPIN>
@@ -794,7 +790,7 @@ cudaError_t launch_wave_fwd(const WaveGeo &g, const float *coeffs, const float *
                             cudaStream_t st, float *lapout)
 {
     StarCoef cf{};
-    for (int i = 0; i < 3 * (2 * g.r + 1); ++i) cf.c[i] = coeffs[i];
+    cf.set(coeffs, 3 * (2 * g.r + 1));
     switch (g.r) {
         case 1: return fwd_r<1>(g, cf, m, p_cur, p_prev, p_next, src_amp, rec, lapout, st);
         case 2: return fwd_r<2>(g, cf, m, p_cur, p_prev, p_next, src_amp, rec, lapout, st);
@@ -809,7 +805,7 @@ cudaError_t launch_wave_adj_scaled(const WaveGeo &g, const float *coeffs, const 
                                    cudaStream_t st)
 {
     StarCoef cf{};
-    for (int i = 0; i < 3 * (2 * g.r + 1); ++i) cf.c[i] = coeffs[i];
+    cf.set(coeffs, 3 * (2 * g.r + 1));
     const AdjArgs adj{resid, lap_a ? grad : nullptr,
                       g.nx % 4 == 0 && g.gss % 4 == 0 && reinterpret_cast<uintptr_t>(grad) % 32 == 0,
                       g.nx % 2 == 0 && reinterpret_cast<uintptr_t>(grad) % 16 == 0};
@@ -828,7 +824,7 @@ cudaError_t launch_wave_adj(const WaveGeo &g, const float *coeffs, const float *
                             cudaStream_t st, bool lapin)
 {
     StarCoef cf{};
-    for (int i = 0; i < 3 * (2 * g.r + 1); ++i) cf.c[i] = coeffs[i];
+    cf.set(coeffs, 3 * (2 * g.r + 1));
 #define MMS_ADJ(R_)                                                                              \
     return lapin ? adj_r<R_, true>(g, cf, m, lam_cur, lam_prev, resid, a_n, grad, st)            \
                  : adj_r<R_, false>(g, cf, m, lam_cur, lam_prev, resid, a_n, grad, st);
