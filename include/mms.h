@@ -120,7 +120,8 @@ typedef struct {
  * The sweep of mms_stencil_apply with explicit pitches, path and tile
  * variant.  The TMA-staged paths need in_pitch_y*4 and in_pitch_z*4 to be
  * multiples of 16 bytes and `in` 16-byte aligned; with MMS_PATH_AUTO an
- * input that breaks this runs on MMS_PATH_NAIVE, with a forced TMA path it
+ * input that breaks this runs on the CUDA cores with plain copies of its
+ * planes instead of TMA (FP32, any pitch), with a forced TMA path it
  * returns MMS_E_ALIGN.  Tensor-core paths support the box and the star of
  * radius 1..4.  The star's variants come in two forms.  The first half
  * (the library's choice) sweep it in one pass: the in-plane x/y part as
@@ -165,8 +166,10 @@ mms_status mms_stencil_apply_host(const mms_stencil_desc *desc, const float *hos
  * measurements compiled into the library: on a device whose name is that of
  * the GPU the table was tuned on, it gives every (shape, radius, path) its
  * measured best variant, and it holds a BF16x3 row only where that path beat
- * the CUDA cores.  Elsewhere AUTO takes the TMA CUDA-core path (the naive
- * path for unaligned input).  Host only; the first call on a device reads
+ * the CUDA cores.  Elsewhere AUTO takes the TMA CUDA-core path.  For unaligned
+ * input the answer is MMS_PATH_NAIVE, the path for any pitch (AUTO stages the
+ * planes by plain copies there; MMS_PATH_NAIVE itself, forced, reads point by
+ * point).  Host only; the first call on a device reads
  * the device's name (cudaGetDeviceProperties). */
 int32_t mms_auto_path(int shape, int radius, int tma_aligned);
 

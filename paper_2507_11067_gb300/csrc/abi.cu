@@ -138,8 +138,10 @@ March plan_march(const Slots &sl, int64_t tiles_x, int64_t tiles_y, int nshots, 
     const int64_t cols = tiles_x * tiles_y * nshots;
     tz = z_chunk(sl, cols, nz, halo, tz, threads);
     *ctas = cols * ((nz + tz - 1) / tz);
-    const int64_t n = (*ctas + sl.sms - 1) / sl.sms;  // CTAs per SM, spread evenly
-    if (n < sl.per_sm) {
+    // CTAs per SM, spread evenly.  Only where they are few: the shared memory
+    // is taken from L1, and a busy SM evens out by itself.
+    const int64_t n = (*ctas + sl.sms - 1) / sl.sms;
+    if (n < sl.per_sm && n <= busy_ctas(sl, threads)) {
         const size_t least = kSmemPerSm / (size_t)(n + 1) - kSmemReserved + 16;  // n + 1 of these do not fit
         if (*smem < least) *smem = least < kSmemPerCta ? least : kSmemPerCta;
     }
@@ -260,7 +262,8 @@ static bool tma_ok(const float *in, int64_t ipy, int64_t ipz)
 // AUTO: the tensor-core BF16x3 path where a tuned variant for it exists
 // (the autotuner records one only where it beats the CUDA-core path; the
 // built-in table carries them for the GPUs it was tuned on), else the TMA
-// CUDA-core path, else the naive path for unaligned pitches.
+// CUDA-core path; unaligned inputs take the path for any pitch (the staged
+// copies of sweep_any.cu, or the naive kernel where they do not fit).
 static int auto_path(int shape, int r, bool aligned)
 {
     if (!aligned) return MMS_PATH_NAIVE;
@@ -305,10 +308,11 @@ static mms_status apply(const mms_stencil_desc *d, const float *in, float *out, 
             reinterpret_cast<cudaStream_t>(stream)};
     int path = d->path;
     const bool aligned = tma_ok(in, ipy, ipz);
+    const bool any = path == MMS_PATH_AUTO && !aligned && any_pitch_ok(s);  // any pitch, by staged copies
     if (path == MMS_PATH_AUTO) path = auto_path(shape, r, aligned);
     if (path == MMS_PATH_NAIVE) {
-        cudaError_t e = launch_naive(s);
-        return e == cudaSuccess ? MMS_OK : cuda_fail(e, "naive sweep launch");
+        cudaError_t e = any ? launch_any(s) : launch_naive(s);
+        return e == cudaSuccess ? MMS_OK : cuda_fail(e, any ? "staged sweep launch" : "naive sweep launch");
     }
     if (!aligned)
         return fail(MMS_E_ALIGN, "TMA path needs a 16-byte aligned input and pitches that are multiples of 4 floats");

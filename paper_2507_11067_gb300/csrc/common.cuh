@@ -68,6 +68,10 @@ cudaError_t launch_plane_cc(const Sweep &s, const CUtensorMap &tmap, int variant
 int plane_cc_variants();
 void plane_cc_box(int r, int v, int *bx, int *by);
 
+// Sweeps of inputs TMA cannot read (sweep_any.cu), and whether the grid is one they take.
+bool any_pitch_ok(const Sweep &s);
+cudaError_t launch_any(const Sweep &s);
+
 // Planar shapes have no z halo.
 __host__ __device__ constexpr bool is_planar(int shape) { return shape == MMS_STAR2D || shape == MMS_BOX2D; }
 
