@@ -101,11 +101,7 @@ cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t
     return cudaSuccess;
 }
 
-// CTAs per SM up to which another one costs an SM nothing: 256 threads are two
-// warps per scheduler, and a plane step of fewer is latency (the radius-4
-// star: 0.49 us for a lone CTA of 128 threads, 0.23 us per CTA when four
-// share the SM); and the CTAs that keep an SM busy (512 threads).
-static int free_ctas(int threads) { return threads < 256 ? 256 / threads : 1; }
+// CTAs that keep an SM busy (512 threads).
 static int busy_ctas(const Slots &sl, int threads)
 {
     const int n = (512 + threads - 1) / threads;
@@ -116,19 +112,33 @@ int z_chunk(const Slots &sl, int64_t cols, int64_t nz, int halo, int tz, int thr
 {
     if (cols < 1 || nz < 1) return tz;
     if (tz > nz) tz = (int)nz;
-    const int busy = busy_ctas(sl, threads), alone = free_ctas(threads);
-    if (cols * ((nz + tz - 1) / tz) >= (int64_t)sl.sms * busy) return tz;
+    if (cols * ((nz + tz - 1) / tz) >= (int64_t)sl.sms * busy_ctas(sl, threads)) return tz;
+    const int most = (1024 + threads - 1) / threads, per = most < sl.per_sm ? most : sl.per_sm;
+    const double slots = (double)sl.sms * per;
+    // steps of a march x the time of a step, in steps of a full SM: a lone
+    // CTA's step is latency and takes 0.4 to 0.5 of that (star r = 4, 256^3:
+    // 0.48, 0.50, 0.65, 0.92 us at 1 to 4 CTAs per SM); more CTAs than slots
+    // run in waves, the last of which overlaps the others' ends
     const auto cost = [&](int64_t t) {
-        const int64_t n = (cols * ((nz + t - 1) / t) + sl.sms - 1) / sl.sms;
-        return (t + halo) * (n > alone ? n : alone);
+        const int64_t c = cols * ((nz + t - 1) / t);
+        return (double)(t + halo) * ((double)c <= slots ? 0.37 + 0.63 * (double)((c + sl.sms - 1) / sl.sms) / per
+                                                        : (double)c / slots + 0.5);
     };
     int64_t best = tz;
-    for (int n = 1; n <= busy; ++n) {
-        const int64_t k = (int64_t)sl.sms * n / cols;  // chunks per column
-        if (k < 1) continue;
+    double least = cost(tz);
+    const auto consider = [&](int64_t ctas) {
+        const int64_t k = ctas / cols;  // chunks per column
+        if (k < 1) return;
         const int64_t t = (nz + k - 1) / k;
-        if (t <= tz && cost(t) < cost(best)) best = t;
-    }
+        if (t > tz) return;             // the tuned chunk is the longest
+        const double c = cost(t);
+        if (c < least) {
+            least = c;
+            best = t;
+        }
+    };
+    for (int n = 1; n <= per; ++n) consider((int64_t)sl.sms * n);  // one wave of n CTAs per SM
+    for (int h = 3; h <= 8; ++h) consider((int64_t)(0.5 * h * slots));  // one and a half to four waves
     return (int)best;
 }
 

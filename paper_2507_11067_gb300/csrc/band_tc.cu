@@ -838,6 +838,29 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
     }
 }
 
+// Output planes per tile, given the variant's `nzt`.  The persistent CTAs
+// (`slots` of them) take whole tiles, so a sweep lasts the most tiles any of
+// them has x the planes of one (halo planes and about four planes' time to
+// fill the pipeline included).  A grid of four tiles per CTA or more keeps the
+// variant's planes (512^3: within 2 % of each other from 32 to 64 planes);
+// below that the depth that makes the product least is taken: box r = 4 on
+// 251 x 190 x 133 has 320 tiles of 32 planes for 304 CTAs, two rounds, or 256
+// of 34, one (68 -> 50 us).
+int tile_planes(int64_t slots, int64_t cols, int64_t nz, int halo, int nzt)
+{
+    if (nzt > nz) nzt = (int)nz;
+    if (cols * ((nz + nzt - 1) / nzt) >= 4 * slots) return nzt;
+    const auto cost = [&](int64_t t) { return (cols * ((nz + t - 1) / t) + slots - 1) / slots * (t + halo + 4); };
+    int64_t best = nzt;
+    for (int rounds = 1; rounds <= 4; ++rounds) {
+        const int64_t k = rounds * slots / cols;  // tiles per column
+        if (k < 1) continue;
+        const int64_t t = (nz + k - 1) / k;
+        if (t <= 128 && cost(t) < cost(best)) best = t;
+    }
+    return (int)best;
+}
+
 // What one launch computes: the band weights (box: (2r+1)^3; planar and
 // star: the (2r+1)^2 in-plane set), the star's z weights, where the staged
 // planes start, and where the results go.
@@ -874,7 +897,7 @@ cudaError_t launch_r(const Sweep &s, const CUtensorMap &map, int nzt, const Laun
     // persistent: one CTA per SM, two for the dual configuration
     sl.per_sm = C::DUAL ? 2 : 1;
     const int64_t tx = (s.nx + C::TX - 1) / C::TX, ty = (s.ny + C::TY - 1) / C::TY;
-    nzt = z_chunk(sl, tx * ty, s.nz, 2 * C::RZ, nzt, C::NT);
+    nzt = tile_planes((int64_t)sl.sms * sl.per_sm, tx * ty, s.nz, 2 * C::RZ, nzt);
     const int64_t tz = (s.nz + nzt - 1) / nzt;
     if (tx * ty * tz > (int64_t)1 << 30) return cudaErrorInvalidValue;
     a.tiles_x = (int)tx;

@@ -115,12 +115,12 @@ cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t
 
 // Planes per z chunk of a kernel whose CTAs each march one chunk of one of
 // `cols` columns (reading `halo` extra planes), given the kernel's tuned chunk
-// `tz`.  A march takes (planes + halo) steps, so a launch that leaves the
-// device half empty takes about (t + halo) x the busiest SM's CTAs; the chunk
-// t is the one that makes this least among those that give an SM 1, 2, ...
-// CTAs.  A grid whose tuned chunks keep every SM busy keeps them: it is bound
+// `tz`.  A grid whose tuned chunks keep every SM busy keeps them: it is bound
 // by memory, and finer chunks only read more halo planes (box r = 1, 512^3:
-// 172 us, 196 us in finer ones).
+// 172 us, 196 us in finer ones).  Otherwise the chunk is the one of least
+// modelled time among those that fill one wave to 1, 2, ... CTAs per SM or run
+// in one and a half to four waves: the VTI step on 2 x 250 x 230 x 190, 232
+// columns on 456 CTA slots, takes 285 us as one chunk each, 174 us in five.
 int z_chunk(const Slots &sl, int64_t cols, int64_t nz, int halo, int tz, int threads);
 
 // How a kernel's CTAs divide the columns they march along z: CTA b marches
