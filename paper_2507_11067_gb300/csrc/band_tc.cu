@@ -240,7 +240,6 @@ struct TcArgs {
     float *out;
     int64_t opy, opz;
     int nx, ny, nz;
-    int vec;                      // output store width: 4 (float4), 2 (float2) or 1
     int tiles_x, tiles_y, tiles;  // tiles = tiles_x * tiles_y * z chunks
     int nzt;                      // output planes per z chunk
     int zoff;                     // padded input plane of staged plane 0 of chunk 0
@@ -308,6 +307,17 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
         ptx::fence_mbar_init();
         *abort_flag = 0;
     }
+    // The weights go to shared memory first (the staging ring is still free):
+    // the band's words index them by lane, and the constant bank serves one
+    // address at a time (box r = 4, 64^3: 20.9 -> 18.0 us).  The pointer is opaque
+    // so that they are read as ordinary memory, a warp at a time.
+    {
+        const float *w = cf.c;
+        asm("" : "+l"(w));
+        constexpr int NC = MODE == M_BOX ? W * W * W : W * W;
+        for (int i = tid; i < NC; i += C::NT) stg[i] = w[i];
+    }
+    __syncthreads();
     // The band operand: 32-bit word w of the band area holds K element(s)
     // k0 (and k0 + 1 for BF16, high half) of band row n of part p of plane
     // offset dz.
@@ -325,13 +335,13 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
         for (int h = 0; h < (C::BF ? 2 : 1); ++h) {
             const int d = k0 + h - xo;
             if (n < C::NB && d >= 0 && d <= 2 * R) {
-                const float c = MODE == M_BOX ? cf.c[(dzi * W + dyi) * W + d] : cf.c[dyi * W + d];
+                const float c = stg[(MODE == M_BOX ? dzi * W + dyi : dyi) * W + d];
                 word |= split_part<PREC>(c, p) << (16 * h);
             }
         }
         reinterpret_cast<uint32_t *>(band)[w] = word;
     }
-    ptx::fence_proxy_async_smem();  // generic writes -> tensor-core reads
+    ptx::fence_proxy_async_smem();  // generic writes -> tensor-core reads (and the weights' reads -> TMA writes)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -677,7 +687,7 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
                 if constexpr (MODE == M_STAR) acc += __uint_as_float(zz[x]);
                 o[x] = acc;
             }
-            const int y = y0 + t, xb = x0 + q * C::TXO, zg = z0 + z;
+            const int xb = x0 + q * C::TXO, zg = z0 + z;
             if constexpr (C::TSTORE) {
                 if (a.tstore) {
                     // the subtile into this warp's buffer for the output's
@@ -704,23 +714,25 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
                     return true;
                 }
             }
-            if (t < C::TY && y < a.ny && xb < a.nx) {
-                float *op = a.out + (int64_t)zg * a.opz + (int64_t)y * a.opy + xb;
-                const bool full = xb + C::TXO <= a.nx;
-                if (C::TXO % 4 == 0 && full && a.vec == 4) {
+            // Outputs whose rows are no 16-byte multiples: the subtile goes
+            // through shared memory and leaves in element order, so that a
+            // store writes whole row pieces instead of one element of each of
+            // 32 rows (box r = 4 on 251 x 190 x 133: 64.7 -> 54.5 us).
+            float *ob = obuf + (size_t)(nout & 1) * (C::OBUF / 4);
+            if (t < C::TY) {
 #pragma unroll
-                    for (int i = 0; i < C::TXO / 4; ++i)
-                        reinterpret_cast<float4 *>(op)[i] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
-                } else if (full && a.vec >= 2) {
-#pragma unroll
-                    for (int i = 0; i < C::TXO / 2; ++i)
-                        reinterpret_cast<float2 *>(op)[i] = make_float2(o[2 * i], o[2 * i + 1]);
-                } else {
-#pragma unroll
-                    for (int x = 0; x < C::TXO; ++x)
-                        if (xb + x < a.nx) op[x] = o[x];
-                }
+                for (int i = 0; i < C::TXO / 4; ++i)
+                    reinterpret_cast<float4 *>(ob + t * C::TXO)[i] =
+                        make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
             }
+            __syncwarp();
+            float *op = a.out + (int64_t)zg * a.opz + (int64_t)y0 * a.opy + xb;
+#pragma unroll
+            for (int i = 0; i < (C::TXO * C::TY + 31) / 32; ++i) {
+                const int e = i * 32 + lane, row = e / C::TXO, x = e % C::TXO;
+                if (row < C::TY && y0 + row < a.ny && xb + x < a.nx) op[(int64_t)row * a.opy + x] = ob[e];
+            }
+            ++nout;  // the other buffer next: its reads ended before this output's __syncwarp
             if (lane == 0 && q == 0) MMS_TL(8, j);
             tep += MMS_CLOCK() - t1;
             return true;
@@ -845,7 +857,7 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
 // variant's planes (512^3: within 2 % of each other from 32 to 64 planes);
 // below that the depth that makes the product least is taken: box r = 4 on
 // 251 x 190 x 133 has 320 tiles of 32 planes for 304 CTAs, two rounds, or 256
-// of 34, one (68 -> 50 us).
+// of 34, one.
 int tile_planes(int64_t slots, int64_t cols, int64_t nz, int halo, int nzt)
 {
     if (nzt > nz) nzt = (int)nz;
@@ -887,8 +899,6 @@ cudaError_t launch_r(const Sweep &s, const CUtensorMap &map, int nzt, const Laun
     a.nx = (int)s.nx;
     a.ny = (int)s.ny;
     a.nz = (int)s.nz;
-    const uintptr_t ob = reinterpret_cast<uintptr_t>(L.out);
-    a.vec = (L.opy % 4 == 0 && L.opz % 4 == 0 && ob % 16 == 0) ? 4 : (L.opy % 2 == 0 && L.opz % 2 == 0 && ob % 8 == 0) ? 2 : 1;
     auto kern = band_tc_kernel<R, PREC, MODE>;
     static SlotCache cache;
     Slots sl;
@@ -908,9 +918,9 @@ cudaError_t launch_r(const Sweep &s, const CUtensorMap &map, int nzt, const Laun
     if (MODE == M_STAR)
         for (int d = 0; d < C::W; ++d) a.cz[d] = L.cz[d];
     // outputs by TMA stores where the subtile rows and the output's pitches
-    // are 16-byte multiples (and the map encodes); else from registers
+    // are 16-byte multiples (and the map encodes); else row piece by row piece
     CUtensorMap omap{};
-    a.tstore = C::TSTORE && a.vec == 4 &&
+    a.tstore = L.opy % 4 == 0 && L.opz % 4 == 0 && reinterpret_cast<uintptr_t>(L.out) % 16 == 0 &&
                encode_tmap_3d(&omap, L.out, s.nx, s.ny, s.nz, L.opy, L.opz, C::TSTORE ? C::TXO : 4, C::TY, 1);
     const int slots = sl.sms * sl.per_sm;
     const int grid = a.tiles < slots ? a.tiles : slots;
