@@ -220,7 +220,10 @@ def _ptr(t) -> ctypes.c_void_p:
 def _stream(stream):
     import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the handle of the current device's current stream, without the Stream
+        # object that torch.cuda.current_stream() builds (0.1 against 3.2 us of
+        # the 17 us a small sweep's call took)
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return ctypes.c_void_p(int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream))
 
 
@@ -233,7 +236,7 @@ def _host_coeffs(coeffs, count=None, dtype=np.float32) -> np.ndarray:
     """The weights as a contiguous host array; with count, refused unless it
     holds exactly that many (the library reads count values)."""
     c = coeffs
-    if hasattr(c, "detach"):
+    if not isinstance(c, np.ndarray) and hasattr(c, "detach"):
         c = c.detach().cpu().numpy()
     c = np.ascontiguousarray(np.asarray(c, dtype=dtype).reshape(-1))
     if count is not None and c.size != count:
