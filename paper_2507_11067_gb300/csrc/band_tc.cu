@@ -717,7 +717,7 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
             // Outputs whose rows are no 16-byte multiples: the subtile goes
             // through shared memory and leaves in element order, so that a
             // store writes whole row pieces instead of one element of each of
-            // 32 rows (box r = 4 on 251 x 190 x 133: 64.7 -> 54.5 us).
+            // 32 rows (box r = 4 on 251 x 190 x 133: 64.7 -> 54.9 us).
             float *ob = obuf + (size_t)(nout & 1) * (C::OBUF / 4);
             if (t < C::TY) {
 #pragma unroll
@@ -727,7 +727,7 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
             }
             __syncwarp();
             float *op = a.out + (int64_t)zg * a.opz + (int64_t)y0 * a.opy + xb;
-#pragma unroll
+#pragma unroll 1  // unrolled, it slows the other path's loop too (box r = 2, 512^3: 279 against 272 us)
             for (int i = 0; i < (C::TXO * C::TY + 31) / 32; ++i) {
                 const int e = i * 32 + lane, row = e / C::TXO, x = e % C::TXO;
                 if (row < C::TY && y0 + row < a.ny && xb + x < a.nx) op[(int64_t)row * a.opy + x] = ob[e];
