@@ -617,43 +617,83 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT, 2)
         if (!plane(j)) return;
 }
 
-__global__ void model_kernel(WaveGeo geo, const float *__restrict__ v, float *__restrict__ m, float s)
+// The pointwise kernels below run over rows of x (blocks of 4 rows, 64 threads
+// along each), so that a point's place costs no division: with one per
+// coordinate and point they took four times HBM's time (256^3: model 94 -> 26
+// us).
+constexpr int kRowThreads = 64, kRowsPerBlock = 4;
+inline int row_blocks(int64_t rows)
 {
-    const int r = geo.r;
-    const int64_t X = geo.nx + 2 * r, Y = geo.ny + 2 * r, Z = geo.nz + 2 * r;
-    const int64_t total = X * Y * Z;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t xx = i % X, yy = (i / X) % Y, zz = i / (X * Y);
-        const int64_t x = xx - r, y = yy - r, z = zz - r;
-        float val = 0.f;
-        if (x >= 0 && x < geo.nx && y >= 0 && y < geo.ny && z >= 0 && z < geo.nz) {
-            const float vv = v[(z * geo.ny + y) * geo.nx + x];
-            val = vv * vv * s;
+    const int64_t b = (rows + kRowsPerBlock - 1) / kRowsPerBlock;
+    return (int)(b < 152 * 32 ? b : 152 * 32);
+}
+
+__global__ void __launch_bounds__(kRowThreads *kRowsPerBlock)
+    model_kernel(const __grid_constant__ WaveGeo geo, const float *__restrict__ v, float *__restrict__ m, float s)
+{
+    const int r = geo.r, X = geo.nx + 2 * r;
+    const int64_t Y = geo.ny + 2 * r, rows = Y * (geo.nz + 2 * r);
+    for (int64_t row = (int64_t)blockIdx.x * kRowsPerBlock + threadIdx.y; row < rows;
+         row += (int64_t)gridDim.x * kRowsPerBlock) {
+        const int64_t zz = row / Y, yy = row - zz * Y, y = yy - r, z = zz - r;
+        const bool inside = y >= 0 && y < geo.ny && z >= 0 && z < geo.nz;
+        const float *vr = v + (z * geo.ny + y) * geo.nx;
+        float *mr = m + zz * geo.pz + yy * geo.py;
+        for (int xx = threadIdx.x; xx < X; xx += kRowThreads) {
+            const int x = xx - r;
+            float val = 0.f;
+            if (inside && x >= 0 && x < geo.nx) {
+                const float vv = vr[x];
+                val = vv * vv * s;
+            }
+            mr[xx] = val;
         }
-        m[zz * geo.pz + yy * geo.py + xx] = val;
     }
 }
 
 // grad[z][y][x] /= m at the interior point (FP64): the scaled adjoint's sum
-// of mu^{n+1} (L a^n) turned into dJ/dm.
-__global__ void divide_m_kernel(WaveGeo geo, const float *__restrict__ m, double *__restrict__ grad)
+// of mu^{n+1} (L a^n) turned into dJ/dm.  GB300's FP64 pipe makes an IEEE
+// division per point the whole cost (256^3: 635 us, HBM's time is 49), so the
+// quotient comes from a reciprocal of the FP32 m, kept as the sum of two FP32
+// values (r + e, 48 bits, worked out on the FP32 pipe), and one FP64
+// correction step: q = g r', q += (g - q m) r', within an ulp of the
+// quotient.  What that cannot serve (m outside 2^-60 .. 2^60, a quotient that
+// is no number of moderate size) divides; the range is read off the bits, on
+// the integer pipe.
+__device__ __forceinline__ double divide_by_float(double g, float m)
+{
+    if (m >= 0x1p-60f && m <= 0x1p60f) {
+        const float r = 1.f / m, e = r * fmaf(-m, r, 1.f);
+        const double md = widen(m), rd = widen(r) + widen(e);
+        const double q = g * rd;
+        const uint32_t hi = (uint32_t)__double2hiint(q), ex = (hi >> 20) & 0x7ffu;
+        if (ex - 123u < 1800u) return fma(fma(-q, md, g), rd, q);  // 2^-900 <= |q| < 2^900
+        if (((uint32_t)__double2hiint(g) << 1 | (uint32_t)__double2loint(g)) == 0u) return g;
+    }
+    return g / (double)m;
+}
+
+__global__ void __launch_bounds__(kRowThreads *kRowsPerBlock)
+    divide_m_kernel(const __grid_constant__ WaveGeo geo, const float *__restrict__ m, double *__restrict__ grad)
 {
     const int r = geo.r;
-    const int64_t n = (int64_t)geo.nx * geo.ny * geo.nz;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t x = i % geo.nx, y = (i / geo.nx) % geo.ny, z = i / ((int64_t)geo.nx * geo.ny);
-        grad[i] = grad[i] / (double)m[(z + r) * geo.pz + (y + r) * geo.py + x + r];
+    const int64_t rows = (int64_t)geo.ny * geo.nz;
+    for (int64_t row = (int64_t)blockIdx.x * kRowsPerBlock + threadIdx.y; row < rows;
+         row += (int64_t)gridDim.x * kRowsPerBlock) {
+        const int64_t z = row / geo.ny, y = row - z * geo.ny;
+        double *gr = grad + row * geo.nx;
+        const float *mr = m + (z + r) * geo.pz + (y + r) * geo.py + r;
+        for (int x = threadIdx.x; x < geo.nx; x += kRowThreads) gr[x] = divide_by_float(gr[x], mr[x]);
     }
 }
 
+// gv = gm 2 v dt^2/h^2; s2 = 2 dt^2/h^2 (a factor of two rounds nothing)
 __global__ void chain_kernel(const double *__restrict__ gm, const float *__restrict__ v,
-                             double *__restrict__ gv, int64_t n, double s)
+                             double *__restrict__ gv, int64_t n, double s2)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
-        gv[i] = gm[i] * 2.0 * (double)v[i] * s;
+        gv[i] = gm[i] * widen(v[i]) * s2;
 }
 
 __global__ void sum_kernel(const double *__restrict__ slices, int nslices, int64_t stride, int64_t n,
@@ -842,7 +882,8 @@ cudaError_t launch_model_from_velocity(const WaveGeo &g, const float *v, float *
                                        cudaStream_t st)
 {
     const float s = (dt * dt) / (h * h);
-    model_kernel<<<152 * 8, 256, 0, st>>>(g, v, m, s);
+    model_kernel<<<row_blocks((int64_t)(g.ny + 2 * g.r) * (g.nz + 2 * g.r)), dim3(kRowThreads, kRowsPerBlock), 0, st>>>(
+        g, v, m, s);
     return cudaGetLastError();
 }
 
@@ -850,13 +891,13 @@ cudaError_t launch_grad_to_velocity(const double *gm, const float *v, double *gv
                                     float h, cudaStream_t st)
 {
     const double s = ((double)dt * dt) / ((double)h * h);
-    chain_kernel<<<152 * 8, 256, 0, st>>>(gm, v, gv, n, s);
+    chain_kernel<<<152 * 8, 256, 0, st>>>(gm, v, gv, n, 2.0 * s);
     return cudaGetLastError();
 }
 
 cudaError_t launch_grad_divide_m(const WaveGeo &g, const float *m, double *grad, cudaStream_t st)
 {
-    divide_m_kernel<<<152 * 8, 256, 0, st>>>(g, m, grad);
+    divide_m_kernel<<<row_blocks((int64_t)g.ny * g.nz), dim3(kRowThreads, kRowsPerBlock), 0, st>>>(g, m, grad);
     return cudaGetLastError();
 }
 
