@@ -22,6 +22,9 @@
 // it) -- so it runs on the forward kernel with no per-plane product and
 // no barrier between forming and reading it; the accumulated gradient is
 // divided by m once at the end (divide_m_kernel).  It needs m > 0.
+#include <type_traits>
+#include <utility>
+
 #include "common.cuh"
 #include "tile.cuh"
 #include "wave.cuh"
@@ -68,19 +71,21 @@ __global__ void wait_selftest_kernel(unsigned long long limit_ns, unsigned *err)
 // position of F's leading one (FP64 reaches far below 2^-149).
 __device__ __forceinline__ double widen(float f)
 {
-    const uint32_t u = __float_as_uint(f);
-    const uint32_t e = (u >> 23) & 0xffu, frac = u & 0x7fffffu;
-    uint64_t d = (uint64_t)(u & 0x80000000u) << 32;
-    if (e == 0xffu) {
-        d |= (uint64_t)0x7ffu << 52 | (uint64_t)frac << 29;
-    } else if (e != 0u) {
-        d |= (uint64_t)(e + 896u) << 52 | (uint64_t)frac << 29;
-    } else if (frac != 0u) {
-        // leading one of F at bit b = 23 - s: f = 1.xxx 2^(-126 - s)
-        const uint32_t sh = (uint32_t)__clz(frac) - 8u;
-        d |= (uint64_t)(897u - sh) << 52 | (uint64_t)((frac << sh) & 0x7fffffu) << 29;
+    const uint32_t u = __float_as_uint(f), a = u & 0x7fffffffu;
+    uint32_t hi = (a >> 3) + (896u << 20), lo = u << 29;
+    if (a - 0x00800000u >= 0x7f000000u) {  // not a normal number
+        if (a >= 0x7f800000u) {
+            hi = 0x7ff00000u | (a & 0x7fffffu) >> 3;
+        } else if (a == 0u) {
+            hi = 0u;
+        } else {
+            // leading one of F at bit b = 23 - s: f = 1.xxx 2^(-126 - s)
+            const uint32_t sh = (uint32_t)__clz(a) - 8u, frac = (a << sh) & 0x7fffffu;
+            hi = (897u - sh) << 20 | frac >> 3;
+            lo = frac << 29;
+        }
     }
-    return __longlong_as_double((long long)d);
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)lo);
 }
 
 // Ring stage s: [a^n plane + halo | m tile | a^{n-1} tile | a^n tile].  The
@@ -93,8 +98,11 @@ __device__ __forceinline__ double widen(float f)
 // update has the forward step's form (the stencil acts on the state itself),
 // with the receiver residual m r^n in place of the source and the FP64
 // gradient term mu^{n+1} (L a^n) = m G lam^{n+1} (L a^n), L a^n read from a
-// fifth tile.
-enum { K_FWD = 0, K_FWD_LAP = 1, K_ADJ_SCALED = 2 };
+// fifth tile -- K_ADJ_BULK where a plane's terms leave by bulk reductions (one
+// shared slice, rows of 16 bytes), K_ADJ for the rest (no gradient, atomics,
+// per-shot slices): the bulk form's registers decide how many CTAs an SM
+// holds, so it carries nothing of the others.
+enum { K_FWD = 0, K_FWD_LAP = 1, K_ADJ = 2, K_ADJ_BULK = 3 };
 
 template <int R, int TX, int TY, int PY, int S, int MODE = K_FWD>
 struct FwdGeom {
@@ -106,11 +114,11 @@ struct FwdGeom {
     static constexpr int OFF_P = OFF_M + ((MT + 31) & ~31);
     static constexpr int OFF_C = OFF_P + ((MT + 31) & ~31);
     static constexpr int OFF_L = OFF_C + ((MT + 31) & ~31);  // adjoint: L a^n
-    static constexpr int STAGE = OFF_L + (MODE == K_ADJ_SCALED ? ((MT + 31) & ~31) : 0);
-    // adjoint: two FP64 buffers of an output plane's gradient terms (TY x
+    static constexpr int STAGE = OFF_L + (MODE >= K_ADJ ? ((MT + 31) & ~31) : 0);
+    // K_ADJ_BULK: two FP64 buffers of an output plane's gradient terms (TY x
     // TX), 128-byte aligned after the ring's barriers and abort flag
     static constexpr size_t OFF_GB = ((size_t)S * STAGE * 4 + S * sizeof(uint64_t) + 16 + 127) / 128 * 128;
-    static constexpr size_t GB_BYTES = MODE == K_ADJ_SCALED ? 2 * (size_t)TY * TX * sizeof(double) : 0;
+    static constexpr size_t GB_BYTES = MODE == K_ADJ_BULK ? 2 * (size_t)TY * TX * sizeof(double) : 0;
     static constexpr size_t SMEM = 128 + OFF_GB + GB_BYTES;
 };
 
@@ -179,7 +187,7 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
                     const __grid_constant__ AdjArgs adj, const __grid_constant__ March march, int vec, unsigned *err)
 {
     constexpr bool LAPOUT = MODE == K_FWD_LAP;
-    constexpr bool ADJ = MODE == K_ADJ_SCALED;
+    constexpr bool ADJ = MODE >= K_ADJ, gbulk = MODE == K_ADJ_BULK;
     using G = Geom<R, TX, TY, PY, S>;
     using F = FwdGeom<R, TX, TY, PY, S, MODE>;
     using I = Interior<R, TX>;
@@ -195,11 +203,10 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
     const int tid = threadIdx.x;
     const int tx = tid % G::NTX, ty = tid / G::NTX;
     const int ry0 = ty * PY;
-    const bool has_grad = ADJ && adj.grad != nullptr;
-    // The shots' terms go to one shared gradient: each output plane's terms
-    // are gathered in shared memory and each row is added by one bulk
+    const bool has_grad = gbulk || (ADJ && adj.grad != nullptr);
+    // gbulk: the shots' terms go to one shared gradient; each output plane's
+    // terms are gathered in shared memory and each row is added by one bulk
     // reduction (the L2 does the adds), instead of one FP64 atomic per point.
-    [[maybe_unused]] const bool gbulk = has_grad && geo.gss == 0 && adj.gbulk;
     [[maybe_unused]] double *gbuf = reinterpret_cast<double *>(smem + F::OFF_GB);
     const int ntiles = has_grad ? 4 : 3;
 
@@ -239,11 +246,18 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
     __syncthreads();
     if (tid == 0)
         for (int j = 0; j < S && j < P; ++j) issue(j);
-    float gxs[4], gys[PY];
+    f2 gxy[PY][2];  // sponge factors g(x) g(y) of the thread's points
+    {
+        float gxs[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) gxs[k] = sponge(gx + k, geo.nx, geo.sponge_w, geo.sponge_a);
+        for (int k = 0; k < 4; ++k) gxs[k] = sponge(gx + k, geo.nx, geo.sponge_w, geo.sponge_a);
 #pragma unroll
-    for (int i = 0; i < PY; ++i) gys[i] = sponge(y0 + ry0 + i, geo.ny, geo.sponge_w, geo.sponge_a);
+        for (int i = 0; i < PY; ++i) {
+            const float gy = sponge(y0 + ry0 + i, geo.ny, geo.sponge_w, geo.sponge_a);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) gxy[i][h] = mul2(pair(gxs[2 * h], gxs[2 * h + 1]), pair(gy, gy));
+        }
+    }
 
     f2 acc[W][PY][2];
 #pragma unroll
@@ -277,7 +291,7 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
         }
         __syncthreads();
         if (abort_flag) {
-            if constexpr (ADJ) bulk_wait_all();  // no reduction still reads this CTA's buffers
+            if constexpr (gbulk) bulk_wait_all();  // no reduction still reads this CTA's buffers
             return;
         }
         if (tid == 0 && j + S < P) issue(j + S);
@@ -287,11 +301,9 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
             // this output plane's gradient buffer; the reductions of the plane
             // before last, which read it, are done first
             [[maybe_unused]] double *gb = gbuf + (size_t)(zo & 1) * (TY * TX);
-            if constexpr (ADJ) {
-                if (gbulk) {
-                    if (tx == 0) bulk_wait_read_1();
-                    __syncwarp();
-                }
+            if constexpr (gbulk) {
+                if (tx == 0) bulk_wait_read_1();
+                __syncwarp();
             }
 #pragma unroll
             for (int i = 0; i < PY; ++i) {
@@ -303,24 +315,36 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
                 unpair(acc[0][i][0], lap[0], lap[1]);
                 unpair(acc[0][i][1], lap[2], lap[3]);
                 [[maybe_unused]] double gd[4] = {0.0, 0.0, 0.0, 0.0};
-                [[maybe_unused]] const bool at_rec = ADJ && adj.resid && z == geo.rec_z;
+                float g[4], v[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float g = gxs[k] * gys[i] * gzv;
-                    float v = 2.f * cv[i][k] + mv[i][k] * lap[k] - g * pv[i][k];
-                    if constexpr (ADJ) {
-                        if (at_rec && gx + k < geo.nx)
-                            v += mv[i][k] * adj.resid[((int64_t)sh * geo.ny + y) * geo.nx + gx + k];
-                        // mu^{n+1} (L a^n) = m G lam^{n+1} (L a^n): m is the same
-                        // at every step, so the sum is divided by it once, at
-                        // the end (mms_grad_divide_m).  The term in FP32 (its
-                        // operands are FP32), accumulated in FP64.
-                        if (has_grad) gd[k] = widen(cv[i][k] * lv[i][k]);
-                    } else {
-                        if (gx + k == sx && y == sy && z == sz) v += samp;
-                    }
-                    res[k] = g * v;
+                for (int h = 0; h < 2; ++h) {
+                    const f2 gg = mul2(gxy[i][h], pair(gzv, gzv));
+                    const f2 c = pair(cv[i][2 * h], cv[i][2 * h + 1]), p = pair(pv[i][2 * h], pv[i][2 * h + 1]);
+                    const f2 t = fma2(pair(mv[i][2 * h], mv[i][2 * h + 1]), acc[0][i][h], add2(c, c));
+                    unpair(gg, g[2 * h], g[2 * h + 1]);
+                    unpair(fma2(pair(-gg.x, -gg.y), p, t), v[2 * h], v[2 * h + 1]);
                 }
+                if constexpr (ADJ) {
+                    if (adj.resid && z == geo.rec_z) {
+                        const float *rs = adj.resid + ((int64_t)sh * geo.ny + y) * geo.nx + gx;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (gx + k < geo.nx) v[k] += mv[i][k] * rs[k];
+                    }
+                    // mu^{n+1} (L a^n) = m G lam^{n+1} (L a^n): m is the same
+                    // at every step, so the sum is divided by it once, at
+                    // the end (mms_grad_divide_m).  The term in FP32 (its
+                    // operands are FP32), accumulated in FP64.
+                    if (has_grad)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) gd[k] = widen(cv[i][k] * lv[i][k]);
+                } else if (z == sz && y == sy) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (gx + k == sx) v[k] += samp;
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) res[k] = g[k] * v[k];
                 if (vec && gx + 3 < geo.nx) {
                     *reinterpret_cast<float4 *>(pp) = make_float4(res[0], res[1], res[2], res[3]);
                 } else {
@@ -747,23 +771,23 @@ cudaError_t fwd_r(const WaveGeo &g, const StarCoef &cf, const float *m, const fl
     } else {
         mlap = mctr;  // not read
     }
-    const int mode = adj ? K_ADJ_SCALED : lapout ? K_FWD_LAP : K_FWD;
-    auto kern = mode == K_ADJ_SCALED ? wave_fwd_kernel<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_ADJ_SCALED>
-                : mode == K_FWD_LAP  ? wave_fwd_kernel<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_FWD_LAP>
-                                     : wave_fwd_kernel<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_FWD>;
-    using FA = FwdGeom<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_ADJ_SCALED>;
-    // the adjoint's gradient buffers only where its bulk reductions run
-    const bool gbulk = adj && adj->grad && g.gss == 0 && adj->gbulk;
-    size_t smem = mode == K_ADJ_SCALED ? FA::SMEM - (gbulk ? 0 : FA::GB_BYTES)
-                        : mode == K_FWD_LAP  ? FwdGeom<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_FWD_LAP>::SMEM
-                                             : FwdGeom<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, K_FWD>::SMEM;
-    static SlotCache caches[4];  // per form (the adjoint without and with its gradient buffers)
+    const int mode = adj ? (adj->grad && g.gss == 0 && adj->gbulk ? K_ADJ_BULK : K_ADJ) : lapout ? K_FWD_LAP : K_FWD;
+    const auto form = [](auto m) {
+        constexpr int M = decltype(m)::value;
+        return std::make_pair(wave_fwd_kernel<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, M>,
+                              FwdGeom<R, kFwdTX, kFwdTY, kFwdPY, kFwdS, M>::SMEM);
+    };
+    auto [kern, smem] = mode == K_ADJ_BULK ? form(std::integral_constant<int, K_ADJ_BULK>{})
+                        : mode == K_ADJ    ? form(std::integral_constant<int, K_ADJ>{})
+                        : mode == K_FWD_LAP ? form(std::integral_constant<int, K_FWD_LAP>{})
+                                            : form(std::integral_constant<int, K_FWD>{});
+    static SlotCache caches[4];  // per form
     Slots sl;
-    cudaError_t e = kernel_slots(caches[mode + (gbulk ? 1 : 0)], reinterpret_cast<const void *>(kern), G::NT, smem, &sl);
+    cudaError_t e = kernel_slots(caches[mode], reinterpret_cast<const void *>(kern), G::NT, smem, &sl);
     if (e != cudaSuccess) return e;
     const int tiles_x = (g.nx + kFwdTX - 1) / kFwdTX, tiles_y = (g.ny + kFwdTY - 1) / kFwdTY;
     int tz = kFwdTZ;
-    if (mode == K_ADJ_SCALED) {
+    if (adj) {
         // The adjoint step on a grid whose tuned chunks fill at most one wave
         // splits z finer, into about three waves, so that the SMs left with
         // one CTA do not idle while the others finish two (2 x 256^3: 219 ->
