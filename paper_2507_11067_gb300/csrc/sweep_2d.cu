@@ -95,10 +95,13 @@ cudaError_t launch_plane(const Sweep &sw, const CUtensorMap &tmap, const Coef &c
 {
     using G = Geom<R, TX, TY, PY, S>;
     auto kern = plane_cc_kernel<R, TX, TY, PY, S, BOX, Coef>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+    static SlotCache cache;
+    Slots sl;
+    cudaError_t e = kernel_slots(cache, reinterpret_cast<const void *>(kern), G::NT, G::SMEM, &sl);
     if (e != cudaSuccess) return e;
-    const int64_t nblocks = (sw.ny + TY - 1) / TY;
-    const dim3 grid((unsigned)((sw.nx + TX - 1) / TX), (unsigned)((nblocks + bpc - 1) / bpc), (unsigned)sw.nz);
+    const int64_t nblocks = (sw.ny + TY - 1) / TY, tiles_x = (sw.nx + TX - 1) / TX;
+    bpc = z_chunk(sl, tiles_x * sw.nz, nblocks, 0, bpc, G::NT);  // fewer blocks per CTA on small planes
+    const dim3 grid((unsigned)tiles_x, (unsigned)((nblocks + bpc - 1) / bpc), (unsigned)sw.nz);
     const int vec = ((sw.opy % 4) == 0 && (sw.opz % 4) == 0 && (reinterpret_cast<uintptr_t>(sw.out) % 16) == 0) ? 1 : 0;
     kern<<<grid, G::NT, G::SMEM, sw.stream>>>(tmap, cf, sw.out, (int)sw.nx, (int)sw.ny, sw.opy, sw.opz, bpc, vec,
                                                device_error_word());
