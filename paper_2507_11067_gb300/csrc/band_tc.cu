@@ -240,6 +240,7 @@ struct TcArgs {
     float *out;
     int64_t opy, opz;
     int nx, ny, nz;
+    int vec;                      // the star's output store width without TMA: 4 (float4), 2 (float2) or 1
     int tiles_x, tiles_y, tiles;  // tiles = tiles_x * tiles_y * z chunks
     int nzt;                      // output planes per z chunk
     int zoff;                     // padded input plane of staged plane 0 of chunk 0
@@ -714,25 +715,48 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
                     return true;
                 }
             }
-            // Outputs whose rows are no 16-byte multiples: the subtile goes
-            // through shared memory and leaves in element order, so that a
-            // store writes whole row pieces instead of one element of each of
-            // 32 rows (box r = 4 on 251 x 190 x 133: 64.7 -> 54.9 us).
-            float *ob = obuf + (size_t)(nout & 1) * (C::OBUF / 4);
-            if (t < C::TY) {
+            if constexpr (MODE == M_STAR) {
+                // from registers: the star's epilogue has none left for the form
+                // below (r = 4, 1024^3, TMA stores: 4.91 ms with this, 5.35 with that)
+                const int y = y0 + t;
+                if (t < C::TY && y < a.ny && xb < a.nx) {
+                    float *op = a.out + (int64_t)zg * a.opz + (int64_t)y * a.opy + xb;
+                    const bool full = xb + C::TXO <= a.nx;
+                    if (C::TXO % 4 == 0 && full && a.vec == 4) {
 #pragma unroll
-                for (int i = 0; i < C::TXO / 4; ++i)
-                    reinterpret_cast<float4 *>(ob + t * C::TXO)[i] =
-                        make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
-            }
-            __syncwarp();
-            float *op = a.out + (int64_t)zg * a.opz + (int64_t)y0 * a.opy + xb;
+                        for (int i = 0; i < C::TXO / 4; ++i)
+                            reinterpret_cast<float4 *>(op)[i] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                    } else if (full && a.vec >= 2) {
+#pragma unroll
+                        for (int i = 0; i < C::TXO / 2; ++i)
+                            reinterpret_cast<float2 *>(op)[i] = make_float2(o[2 * i], o[2 * i + 1]);
+                    } else {
+#pragma unroll
+                        for (int x = 0; x < C::TXO; ++x)
+                            if (xb + x < a.nx) op[x] = o[x];
+                    }
+                }
+            } else {
+                // Outputs whose rows are no 16-byte multiples: the subtile goes
+                // through shared memory and leaves in element order, so that a
+                // store writes whole row pieces instead of one element of each of
+                // 32 rows (box r = 4 on 251 x 190 x 133: 64.7 -> 54.9 us).
+                float *ob = obuf + (size_t)(nout & 1) * (C::OBUF / 4);
+                if (t < C::TY) {
+#pragma unroll
+                    for (int i = 0; i < C::TXO / 4; ++i)
+                        reinterpret_cast<float4 *>(ob + t * C::TXO)[i] =
+                            make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+                }
+                __syncwarp();
+                float *op = a.out + (int64_t)zg * a.opz + (int64_t)y0 * a.opy + xb;
 #pragma unroll 1  // unrolled, it slows the other path's loop too (box r = 2, 512^3: 279 against 272 us)
-            for (int i = 0; i < (C::TXO * C::TY + 31) / 32; ++i) {
-                const int e = i * 32 + lane, row = e / C::TXO, x = e % C::TXO;
-                if (row < C::TY && y0 + row < a.ny && xb + x < a.nx) op[(int64_t)row * a.opy + x] = ob[e];
+                for (int i = 0; i < (C::TXO * C::TY + 31) / 32; ++i) {
+                    const int e = i * 32 + lane, row = e / C::TXO, x = e % C::TXO;
+                    if (row < C::TY && y0 + row < a.ny && xb + x < a.nx) op[(int64_t)row * a.opy + x] = ob[e];
+                }
+                ++nout;  // the other buffer next: its reads ended before this output's __syncwarp
             }
-            ++nout;  // the other buffer next: its reads ended before this output's __syncwarp
             if (lane == 0 && q == 0) MMS_TL(8, j);
             tep += MMS_CLOCK() - t1;
             return true;
@@ -920,7 +944,9 @@ cudaError_t launch_r(const Sweep &s, const CUtensorMap &map, int nzt, const Laun
     // outputs by TMA stores where the subtile rows and the output's pitches
     // are 16-byte multiples (and the map encodes); else row piece by row piece
     CUtensorMap omap{};
-    a.tstore = L.opy % 4 == 0 && L.opz % 4 == 0 && reinterpret_cast<uintptr_t>(L.out) % 16 == 0 &&
+    const uintptr_t ob = reinterpret_cast<uintptr_t>(L.out);
+    a.vec = (L.opy % 4 == 0 && L.opz % 4 == 0 && ob % 16 == 0) ? 4 : (L.opy % 2 == 0 && L.opz % 2 == 0 && ob % 8 == 0) ? 2 : 1;
+    a.tstore = a.vec == 4 &&
                encode_tmap_3d(&omap, L.out, s.nx, s.ny, s.nz, L.opy, L.opz, C::TSTORE ? C::TXO : 4, C::TY, 1);
     const int slots = sl.sms * sl.per_sm;
     const int grid = a.tiles < slots ? a.tiles : slots;
