@@ -78,9 +78,10 @@ class WavePropagator:
         (n_ckpt, 2, field elements): (a^k, a^{k-1}) at k = j*ckpt_every."""
         self.set_velocity(v)
         for f in self.p:
-            # the whole storage in one run: the pitched view's fill writes row
-            # by row at a third of HBM's rate
-            self.flat(f).zero_()
+            # the whole storage in one run (where it is the field's own): the
+            # pitched view's fill writes row by row at a third of HBM's rate
+            own = f.untyped_storage().nbytes() == 4 * self.field_elems
+            (self.flat(f) if own else f).zero_()
         amps = amps.to(self.device, torch.float32).contiguous()
         rec = torch.empty((nsteps, self.nshots, self.ny, self.nx), device=self.device)
         ckpt = None
