@@ -19,7 +19,8 @@
 //    per-plane stencils).
 // Weights are kernel parameters, i.e. uniform constant-bank operands of the
 // FMAs.  The naive kernel (one thread per point, global loads) serves any
-// pitch and is the reference path of the library's own tests.
+// pitch and is the reference path of the library's own tests; AUTO stages the
+// inputs TMA cannot read by plain copies (sweep_any.cu).
 #include <stdio.h>
 
 #include "sweep_cc.cuh"
