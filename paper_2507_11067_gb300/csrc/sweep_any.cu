@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
         if constexpr (BOX)
             box2d_tile<R, PY, G::BX, G::NV>(stages + j % S * G::STAGE, cf, o, tx, ry0);
         else
-            star2d_tile<R, PY, G::BX, G::NV>(stages + j % S * G::STAGE, cf, o, tx, ry0);
+            star2d_tile<R, PY, G::BX, G::NV, true>(stages + j % S * G::STAGE, cf, o, tx, ry0);
         store_rows<PY>(o, out, opy, y0 + j * TY + ry0, ny, gx, nx, vec);
     }
 }

@@ -106,20 +106,25 @@ __device__ __forceinline__ void fma_pair(const W2 &w, const f2 &v, f2 &acc)
     }
 }
 
-// acc (points 0..3 as two pairs) += sum_d w[d + R] * row[k + R + d], d
-// ascending, over the 4 points k of a window row.  A tap whose columns start
-// on an even register pairs with its neighbour.
+// acc (points 2h, 2h + 1) += w[d + R] * row[k + R + d]: tap d of the points'
+// window row.  A tap whose columns start on an even register pairs with its
+// neighbour.
+template <int R>
+__device__ __forceinline__ void tap_x(const W2 *w, const float *row, int d, int h, f2 &acc)
+{
+    const f2 v = pair(row[2 * h + R + d], row[2 * h + R + d + 1]);
+    if (kPairs<R> && (R + d) % 2 == 0) fma_pair<true>(w[d + R], v, acc);
+    else fma_pair<false>(w[d + R], v, acc);
+}
+
+// The four points' x line: every tap, d ascending.
 template <int R>
 __device__ __forceinline__ void line_x(const W2 *w, const float *row, f2 (&acc)[2])
 {
 #pragma unroll
     for (int d = -R; d <= R; ++d)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const f2 v = pair(row[2 * h + R + d], row[2 * h + R + d + 1]);
-            if (kPairs<R> && (R + d) % 2 == 0) fma_pair<true>(w[d + R], v, acc[h]);
-            else fma_pair<false>(w[d + R], v, acc[h]);
-        }
+        for (int h = 0; h < 2; ++h) tap_x<R>(w, row, d, h, acc[h]);
 }
 
 // The centre values (columns R..R+3) of a staged row, as two pairs.
@@ -198,8 +203,10 @@ __device__ __forceinline__ void box_plane(const float *pl, const BoxCoef &cf, f2
 }
 
 // Planar star (Table I's 2D kernels): the thread's 4 x PY outputs of a staged
-// tile, x line (weights c[0..2R]) plus y line (weights c[2R+1..4R+1]).
-template <int R, int PY, int BX, int NV>
+// tile, x line (weights c[0..2R]) plus y line (weights c[2R+1..4R+1]); line
+// after line, or (BY_TAP) tap d of both lines before tap d + 1, the order of
+// the point-by-point kernel.
+template <int R, int PY, int BX, int NV, bool BY_TAP = false>
 __device__ __forceinline__ void star2d_tile(const float *pl, const StarCoef &cf, f2 (&o)[PY][2], int tx, int ry0)
 {
     constexpr int W = 2 * R + 1;
@@ -211,11 +218,14 @@ __device__ __forceinline__ void star2d_tile(const float *pl, const StarCoef &cf,
         float win[4 * NV];
         load_row<NV>(pl + (ry0 + R + i) * BX + 4 * tx, win);
         o[i][0] = o[i][1] = zero2();
-        line_x<R>(cf.c, win, o[i]);
+        if constexpr (!BY_TAP) line_x<R>(cf.c, win, o[i]);
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int d = -R; d <= R; ++d) fma_pair<kPairs<R> && R % 2 == 0>(cf.c[W + d + R], cen[i + R + d][h], o[i][h]);
+            for (int d = -R; d <= R; ++d) {
+                if constexpr (BY_TAP) tap_x<R>(cf.c, win, d, h, o[i][h]);
+                fma_pair<kPairs<R> && R % 2 == 0>(cf.c[W + d + R], cen[i + R + d][h], o[i][h]);
+            }
     }
 }
 
