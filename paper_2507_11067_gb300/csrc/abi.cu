@@ -80,24 +80,33 @@ bool encode_tmap_4d(CUtensorMap *map, const float *base, int64_t X, int64_t Y, i
 }
 
 // ------------------------------------------------------- launch shapes
+unsigned long long context_id()
+{
+    static PFN_cuCtxGetId_v12000 fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<PFN_cuCtxGetId_v12000>(p);
+    });
+    unsigned long long id = 0;
+    return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
 cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t smem, Slots *out)
 {
-    int dev = 0;
+    if (cache.find(context_id(), out)) return cudaSuccess;
+    int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const bool cached = dev >= 0 && dev < SlotCache::kDevs;
-    if (const uint32_t w = cached ? cache.v[dev].load(std::memory_order_acquire) : 0u) {
-        *out = Slots{(int)(w >> 8), (int)(w & 255u)};
-        return cudaSuccess;
-    }
-    int sms = 0, per_sm = 0;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPerCta);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPerCta);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
     if (e != cudaSuccess) return e;
-    if (sms < 1 || per_sm < 1 || per_sm > 255) return cudaErrorInvalidConfiguration;
+    if (sms < 1 || per_sm < 1) return cudaErrorInvalidConfiguration;
     *out = Slots{sms, per_sm};
-    if (cached) cache.v[dev].store((uint32_t)sms << 8 | (uint32_t)per_sm, std::memory_order_release);
+    cache.keep(context_id(), *out);  // (the first call of a process makes its context on the way)
     return cudaSuccess;
 }
 

@@ -7,7 +7,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
+#include <mutex>
 
 #include "../../include/mms.h"
 
@@ -101,16 +101,54 @@ bool encode_tmap_4d(CUtensorMap *map, const float *base, int64_t X, int64_t Y, i
 // a CTA may ask for (sm_103).
 constexpr size_t kSmemPerSm = 228 * 1024, kSmemReserved = 1024, kSmemPerCta = 227 * 1024;
 
-// What one kernel instance can keep resident on a device, asked once per
-// device (with its dynamic shared-memory limit raised to the most there is):
-// the SM count and the CTAs of `threads` threads and `smem` bytes one SM
+// Id of the calling thread's current context, 0 if there is none yet.  A
+// kernel's attributes and the address of a __device__ variable belong to a
+// context, not to a device: what is remembered of them is kept by this id,
+// which no later context has again (not the device's own after a reset either).
+unsigned long long context_id();
+
+// What was worked out last in each of a few contexts (the oldest gives way).
+template <typename T>
+class PerContext {
+public:
+    bool find(unsigned long long ctx, T *out)
+    {
+        std::lock_guard<std::mutex> lk(mu_);
+        for (const Entry &e : e_)
+            if (ctx != 0 && e.ctx == ctx) {
+                *out = e.v;
+                return true;
+            }
+        return false;
+    }
+    void keep(unsigned long long ctx, const T &v)
+    {
+        if (ctx == 0) return;
+        std::lock_guard<std::mutex> lk(mu_);
+        for (const Entry &e : e_)
+            if (e.ctx == ctx) return;  // another thread was first
+        e_[next_] = Entry{ctx, v};
+        next_ = (next_ + 1) % kContexts;
+    }
+
+private:
+    static constexpr int kContexts = 16;
+    struct Entry {
+        unsigned long long ctx = 0;
+        T v{};
+    };
+    std::mutex mu_;
+    Entry e_[kContexts];
+    int next_ = 0;
+};
+
+// What one kernel instance can keep resident on the current device, asked once
+// per context (with its dynamic shared-memory limit raised to the most there
+// is): the SM count and the CTAs of `threads` threads and `smem` bytes one SM
 // holds.  One static cache per kernel instance and size; concurrent first
 // calls compute the same values.
-struct SlotCache {
-    static constexpr int kDevs = 64;
-    std::atomic<uint32_t> v[kDevs];  // SMs << 8 | CTAs per SM, 0 = not asked yet
-};
 struct Slots { int sms = 0, per_sm = 0; };
+using SlotCache = PerContext<Slots>;
 cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t smem, Slots *out);
 
 // Planes per z chunk of a kernel whose CTAs each march one chunk of one of

@@ -35,15 +35,14 @@ __device__ unsigned g_error_word = 0;
 
 unsigned *device_error_word()
 {
-    static unsigned *addr[64] = {nullptr};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-    if (!addr[dev]) {
-        void *p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_error_word) != cudaSuccess) return nullptr;
-        addr[dev] = static_cast<unsigned *>(p);
-    }
-    return addr[dev];
+    static PerContext<unsigned *> cache;
+    unsigned *addr = nullptr;
+    if (cache.find(context_id(), &addr)) return addr;
+    void *p = nullptr;
+    if (cudaGetSymbolAddress(&p, g_error_word) != cudaSuccess) return nullptr;
+    addr = static_cast<unsigned *>(p);
+    cache.keep(context_id(), addr);
+    return addr;
 }
 
 namespace {
