@@ -311,8 +311,11 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
     // The weights go to shared memory first (the staging ring is still free):
     // the band's words index them by lane, and the constant bank serves one
     // address at a time (box r = 4, 64^3: 20.9 -> 18.0 us).  The pointer is opaque
-    // so that they are read as ordinary memory, a warp at a time.
-    {
+    // so that they are read as ordinary memory, a warp at a time.  Not the
+    // star's: its band is one plane's, and the copy costs its epilogue registers
+    // (16 bytes more spilled at r = 4: 1024^3 4.88 -> 5.00 ms, 512^3 660 -> 667 us).
+    constexpr bool WSMEM = MODE != M_STAR;
+    if constexpr (WSMEM) {
         const float *w = cf.c;
         asm("" : "+l"(w));
         constexpr int NC = MODE == M_BOX ? W * W * W : W * W;
@@ -336,7 +339,8 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
         for (int h = 0; h < (C::BF ? 2 : 1); ++h) {
             const int d = k0 + h - xo;
             if (n < C::NB && d >= 0 && d <= 2 * R) {
-                const float c = stg[(MODE == M_BOX ? dzi * W + dyi : dyi) * W + d];
+                const int i = (MODE == M_BOX ? dzi * W + dyi : dyi) * W + d;
+                const float c = WSMEM ? stg[i] : cf.c[i];
                 word |= split_part<PREC>(c, p) << (16 * h);
             }
         }
@@ -717,7 +721,7 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
             }
             if constexpr (MODE == M_STAR) {
                 // from registers: the star's epilogue has none left for the form
-                // below (r = 4, 1024^3, TMA stores: 4.91 ms with this, 5.35 with that)
+                // below (r = 4, 1024^3, TMA stores: 4.88 ms with this, 5.35 with that)
                 const int y = y0 + t;
                 if (t < C::TY && y < a.ny && xb < a.nx) {
                     float *op = a.out + (int64_t)zg * a.opz + (int64_t)y * a.opy + xb;
