@@ -756,6 +756,78 @@ __global__ void dot_kernel(const float *__restrict__ a, const float *__restrict_
 constexpr int kFwdTX = 64, kFwdTY = 16, kFwdPY = 1, kFwdS = 3, kFwdTZ = 128;
 constexpr int kAdjTX = 64, kAdjTY = 16, kAdjS = 2, kAdjTZ = 128;
 
+// The march of a forward step (with L a^n out, `lap`, or without): the planes
+// per CTA and the CTAs an SM may hold (*smem is raised to keep more off it)
+// whose modelled time is least.  `filled`: the part of the tiles' points that
+// are inside the grid.
+//
+// A plane step takes 0.69, 0.93, 1.16 us with one, two, three CTAs on an SM.
+// The form that writes L a^n as well takes 0.72, 1.0, 1.33 us, and from 8 M
+// points on (no longer served by L2) memory holds it up where the third CTA
+// has whole tiles to do: 1.78 us at 95 % of the slots with points, 1.46 at 84
+// %, 1.33 at 75 % (1 x 512^3: 519 us on two CTAs per SM, 568 on three).  CTAs
+// of one length run in waves, a last wave that is not full hardly faster; a
+// short last chunk fills the slots which that wave leaves, or runs after it.
+// The scheduler does not spread the CTAs of one wave by itself: it may put the
+// long ones on some SMs three at a time while others take the short ones (4 x
+// 128 x 200 x 300 in chunks of 128, 128 and 44: 147 us, 117 with two per SM;
+// in four of 75, 93).  Measured over 46 shapes of 1 to 8 shots, the plans take
+// 0.5 % more time than the best ones (lap 1.8 %).  Over 110 others they take
+// 0.50 of the time of 128 planes and two CTAs everywhere (lap 0.54), at most
+// 0.97 (lap 1.06).
+March plan_forward(const Slots &sl, int64_t tiles_x, int64_t tiles_y, const WaveGeo &g, int halo, int tz, bool lap,
+                   double filled, size_t *smem, int64_t *ctas)
+{
+    const int64_t nz = g.nz, cols = tiles_x * tiles_y * g.nshots;
+    const bool big = (double)g.nx * g.ny * (double)nz * g.nshots >= 8e6;
+    // us of a plane step with `n` CTAs per SM of which `inflight` have work
+    const auto step = [&](int n, int64_t inflight) {
+        if (!lap) return 0.69 + 0.235 * (n - 1);
+        if (n <= 2) return n == 1 ? 0.72 : 1.0;
+        const double points = filled * (double)inflight / (double)(sl.sms * 3);
+        return 1.33 * n / 3 + (big && points > 0.7 ? 1.5 * (points - 0.7) : 0.0);
+    };
+    if (tz > nz) tz = (int)nz;
+    int64_t best = tz;
+    int cap = sl.per_sm;
+    double least = 1e300;
+    const auto consider = [&](int64_t t) {
+        if (t < 1 || t > tz) return;  // the tuned chunk is the longest
+        int64_t full = cols * (nz / t), rem = nz % t;
+        if (2 * rem > t) {  // all but as long as the others
+            full += cols;
+            rem = 0;
+        }
+        const double len = (double)(t + halo);
+        for (int c = 1; c <= sl.per_sm; ++c) {
+            const int64_t slots = (int64_t)sl.sms * c, waves = (full + slots - 1) / slots;
+            double cost = waves == 1 ? len * step(c, full)
+                                     : (0.8 * (double)waves + 0.2 * (double)full / (double)slots) * len * step(c, slots);
+            if (rem) {
+                const int64_t left = cols - (waves * slots - full) * ((t + halo) / (rem + halo));
+                if (left > 0)
+                    cost += ((double)left / (double)slots + 0.3) * (double)(rem + halo) *
+                            step(c, left < slots ? left : slots);
+            }
+            if (cost < least) {
+                least = cost;
+                best = t;
+                cap = c;
+            }
+        }
+    };
+    consider(tz);
+    for (int k = 1; k <= 24; ++k) consider((nz + k - 1) / k);
+    for (int c = 1; c <= sl.per_sm; ++c)  // few columns: one wave of c CTAs per SM
+        if (const int64_t k = (int64_t)sl.sms * c / cols; k > 24) consider((nz + k - 1) / k);
+    *ctas = cols * ((nz + best - 1) / best);
+    if (cap < sl.per_sm) {
+        const size_t room = kSmemPerSm / (size_t)(cap + 1) - kSmemReserved + 16;  // cap + 1 of these do not fit
+        if (*smem < room) *smem = room < kSmemPerCta ? room : kSmemPerCta;
+    }
+    return March{(int)tiles_x, (int)tiles_y, g.nshots, (int)best};
+}
+
 template <int R>
 cudaError_t fwd_r(const WaveGeo &g, const StarCoef &cf, const float *m, const float *p_cur,
                   const float *p_prev, float *p_next, const float *amp, float *rec, float *lapout,
@@ -805,7 +877,10 @@ cudaError_t fwd_r(const WaveGeo &g, const StarCoef &cf, const float *m, const fl
         }
     }
     int64_t ctas;
-    const March march = plan_march(sl, tiles_x, tiles_y, g.nshots, g.nz, 2 * R, tz, G::NT, &smem, &ctas);
+    const March march =
+        adj ? plan_march(sl, tiles_x, tiles_y, g.nshots, g.nz, 2 * R, tz, G::NT, &smem, &ctas)
+            : plan_forward(sl, tiles_x, tiles_y, g, 2 * R, tz, mode == K_FWD_LAP,
+                           (double)g.nx * g.ny / ((double)tiles_x * kFwdTX * (double)tiles_y * kFwdTY), &smem, &ctas);
     if (ctas > INT32_MAX) return cudaErrorInvalidConfiguration;
     const int vec = (R % 4 == 0) && g.py % 4 == 0 && g.pz % 4 == 0 && g.ss % 4 == 0 &&
                     reinterpret_cast<uintptr_t>(p_next) % 16 == 0 && reinterpret_cast<uintptr_t>(lapout) % 16 == 0;
