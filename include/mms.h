@@ -174,7 +174,9 @@ mms_status mms_stencil_apply_host(const mms_stencil_desc *desc, const float *hos
 int32_t mms_auto_path(int shape, int radius, int tma_aligned);
 
 /* Number of tile variants of (shape, radius, path); variant indices run
- * 0..n-1.  Returns 0 for an unsupported combination.  Host only. */
+ * 0..n-1.  Returns 0 for an unsupported combination.  A variant is a tile, its
+ * ring and the most planes (row blocks) per thread block; small grids take
+ * fewer (mms_last_planes), also where the variant is named.  Host only. */
 int32_t mms_num_variants(int shape, int radius, int path);
 
 /* Library choice of variant for (shape, radius, path, nx, ny, nz): the one
@@ -527,6 +529,13 @@ mms_status mms_selftest_timeout(uint32_t limit_us, void *stream);
  * without a tensor-core sweep, or a null cfg with ncfg > 0.
  */
 int32_t mms_tc_pipeline_config(int32_t shape, int32_t radius, int32_t path, int32_t *cfg, int32_t ncfg);
+
+/* Output planes (planar shapes: row blocks) that a thread block of the last
+ * tiled sweep (point-by-point and FP64 ones aside) or wave, VTI or TTI step
+ * which this thread queued takes at most; 0 before the first.  Grids that would leave SMs idle are divided finer than
+ * their variant's tile says, so a test of a tile's steady state checks here
+ * that its grid is large enough.  Host only. */
+int32_t mms_last_planes(void);
 
 /* Library version string. */
 const char *mms_version(void);

@@ -9,7 +9,7 @@ loudly if the library has not been built.
 """
 from ._lib import (BOX, BOX2D, PATHS, STAR, STAR2D, MMSError, apply, grad_divide_m, apply_dense, apply_f64, apply_host, auto_path, check_device,
                    default_variant,
-                   dot_f64, field_geometry, grad_to_velocity, load, model_from_velocity,
+                   dot_f64, field_geometry, grad_to_velocity, last_planes, load, model_from_velocity,
                    num_variants, padded_empty, padded_empty2d, pitches, set_variant, sum_f64, tc_pipeline_config,
                    to_padded_device, to_padded_device2d,
                    version, vti_model, vti_step, wave_adjoint, wave_adjoint_lap, wave_adjoint_scaled, wave_desc, wave_forward, wave_step,
@@ -19,7 +19,7 @@ from .build import build
 
 __all__ = ["BOX", "BOX2D", "PATHS", "STAR", "STAR2D", "MMSError", "apply", "grad_divide_m", "apply_dense", "apply_f64", "apply_host", "auto_path", "build",
            "check_device",
-           "default_variant", "dot_f64", "field_geometry", "grad_to_velocity", "load",
+           "default_variant", "dot_f64", "field_geometry", "grad_to_velocity", "last_planes", "load",
            "model_from_velocity", "num_variants", "padded_empty", "padded_empty2d", "pitches", "set_variant", "sum_f64",
            "tc_pipeline_config",
            "to_padded_device", "to_padded_device2d", "version", "wave_adjoint", "wave_desc", "wave_forward", "wave_step",

@@ -191,6 +191,7 @@ def load():
             "mms_aniso_num_variants": [i32],
             "mms_aniso_set_variant": [i32, i32],
             "mms_last_error": [],
+            "mms_last_planes": [],
             "mms_check_device": [P],
             "mms_version": [],
         }
@@ -418,6 +419,11 @@ def default_variant(shape, r, path, nx=0, ny=0, nz=0) -> int:
 
 def set_variant(shape, r, path, variant):
     check(load().mms_set_variant(SHAPES[shape], r, PATHS[path], int(variant)))
+
+
+def last_planes() -> int:
+    """mms_last_planes: planes (row blocks) per thread block of this thread's last launch."""
+    return int(load().mms_last_planes())
 
 
 def check_device(stream=None):

@@ -110,6 +110,9 @@ cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t
     return cudaSuccess;
 }
 
+static thread_local int32_t g_last_planes = 0;
+void note_planes(int64_t planes) { g_last_planes = (int32_t)planes; }
+
 // CTAs that keep an SM busy (512 threads).
 static int busy_ctas(const Slots &sl, int threads)
 {
@@ -164,6 +167,7 @@ March plan_march(const Slots &sl, int64_t tiles_x, int64_t tiles_y, int nshots, 
         const size_t least = kSmemPerSm / (size_t)(n + 1) - kSmemReserved + 16;  // n + 1 of these do not fit
         if (*smem < least) *smem = least < kSmemPerCta ? least : kSmemPerCta;
     }
+    note_planes(tz);
     return March{(int)tiles_x, (int)tiles_y, nshots, tz};
 }
 
@@ -602,6 +606,8 @@ mms_status mms_set_variant(int shape, int radius, int path, int32_t variant)
 }
 
 const char *mms_last_error(void) { return g_last_error.c_str(); }
+
+int32_t mms_last_planes(void) { return g_last_planes; }
 
 const char *mms_version(void) { return "mms-gb300 0.1 (sm_103a)"; }
 

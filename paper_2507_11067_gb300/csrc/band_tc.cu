@@ -942,6 +942,7 @@ cudaError_t launch_r(const Sweep &s, const CUtensorMap &map, int nzt, const Laun
     a.tiles_y = (int)ty;
     a.tiles = (int)(tx * ty * tz);
     a.nzt = nzt;
+    note_planes(nzt);
     a.zoff = L.zoff;
     if (MODE == M_STAR)
         for (int d = 0; d < C::W; ++d) a.cz[d] = L.cz[d];

@@ -177,6 +177,9 @@ struct March {
 March plan_march(const Slots &sl, int64_t tiles_x, int64_t tiles_y, int nshots, int64_t nz, int halo, int tz,
                  int threads, size_t *smem, int64_t *ctas);
 
+// Keeps the planes (row blocks) per CTA of a launch for mms_last_planes.
+void note_planes(int64_t planes);
+
 // The tile, shot and z chunk of this CTA.
 struct Leg {
     int tx, ty, shot, zc;

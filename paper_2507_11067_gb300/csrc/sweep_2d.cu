@@ -101,6 +101,7 @@ cudaError_t launch_plane(const Sweep &sw, const CUtensorMap &tmap, const Coef &c
     if (e != cudaSuccess) return e;
     const int64_t nblocks = (sw.ny + TY - 1) / TY, tiles_x = (sw.nx + TX - 1) / TX;
     bpc = z_chunk(sl, tiles_x * sw.nz, nblocks, 0, bpc, G::NT);  // fewer blocks per CTA on small planes
+    note_planes(bpc);
     const dim3 grid((unsigned)tiles_x, (unsigned)((nblocks + bpc - 1) / bpc), (unsigned)sw.nz);
     const int vec = ((sw.opy % 4) == 0 && (sw.opz % 4) == 0 && (reinterpret_cast<uintptr_t>(sw.out) % 16) == 0) ? 1 : 0;
     kern<<<grid, G::NT, G::SMEM, sw.stream>>>(tmap, cf, sw.out, (int)sw.nx, (int)sw.ny, sw.opy, sw.opz, bpc, vec,

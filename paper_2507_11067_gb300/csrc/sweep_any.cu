@@ -229,6 +229,7 @@ cudaError_t launch_2d(const Sweep &s, const Coef &cf)
     if (e != cudaSuccess) return e;
     const int64_t tiles_x = (s.nx + TX - 1) / TX, tiles_y = (s.ny + TY - 1) / TY;
     const int blocks = z_chunk(sl, tiles_x * s.nz, tiles_y, 0, 8, G::NT);
+    note_planes(blocks);
     const dim3 grid((unsigned)tiles_x, (unsigned)((tiles_y + blocks - 1) / blocks), (unsigned)s.nz);
     const int vec = s.opy % 4 == 0 && s.opz % 4 == 0 && reinterpret_cast<uintptr_t>(s.out) % 16 == 0;
     kern<<<grid, G::NT, G::SMEM, s.stream>>>(s.in, (int)s.ipy, s.ipz, cf, s.out, (int)s.nx, (int)s.ny, s.opy, s.opz,

@@ -825,6 +825,7 @@ March plan_forward(const Slots &sl, int64_t tiles_x, int64_t tiles_y, const Wave
         const size_t room = kSmemPerSm / (size_t)(cap + 1) - kSmemReserved + 16;  // cap + 1 of these do not fit
         if (*smem < room) *smem = room < kSmemPerCta ? room : kSmemPerCta;
     }
+    note_planes(best);
     return March{(int)tiles_x, (int)tiles_y, g.nshots, (int)best};
 }
 
@@ -918,6 +919,7 @@ cudaError_t adj_r(const WaveGeo &g, const StarCoef &cf, const float *m, const fl
     if (e != cudaSuccess) return e;
     const int tiles_x = (g.nx + kAdjTX - 1) / kAdjTX, tiles_y = (g.ny + kAdjTY - 1) / kAdjTY;
     const int tz = z_chunk(sl, (int64_t)tiles_x * tiles_y * g.nshots, g.nz, 2 * R, kAdjTZ, G::NT);
+    note_planes(tz);
     const int nzc = (g.nz + tz - 1) / tz;
     const dim3 grid(tiles_x, tiles_y, nzc * g.nshots);
     // 32-byte aligned rows of four doubles: two double2 per thread

@@ -6,7 +6,9 @@ the fastest is registered with mms_set_variant (so MMS_PATH_AUTO and
 variant -1 use it) and recorded in a JSON table keyed by GPU name, shape,
 radius, path and grid size.  The committed table ``tuned.json`` is loaded by
 ``load_table()``; the paper picks a tile size per kernel by hand (Table I),
-this picks it by measurement.
+this picks it by measurement.  Tune on a grid that keeps every SM busy: smaller
+ones are divided finer than a variant's planes per block (mms_last_planes), so
+variants that differ in nothing else run the same launch there.
 """
 from __future__ import annotations
 
