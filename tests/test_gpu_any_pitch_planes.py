@@ -43,3 +43,21 @@ def test_planar_star_adds_tap_by_tap(r):
         X = nx + 2 * r
         for base, py in ((1, X), (0, X | 1), (2, X + X % 2)):
             assert same_as_naive("star2d", r, c, unaligned(grid, base, py)), (nx, ny, nz, base, py)
+
+
+@pytest.mark.parametrize("shape", ["star2d", "box2d"])
+@pytest.mark.parametrize("r", [1, 2, 3, 4])
+def test_planes_of_many_row_blocks(shape, r):
+    # 35 row blocks in groups of eight, the last group of three and its last
+    # block of 23 rows: ring stages are refilled and the copy re-aimed in mid-march
+    nx, ny, nz = 4090 - r, 1111, 10
+    X = nx + 2 * r
+    c = workloads.normal_coeffs(shape, r, workload=2, salt=50 + r)
+    grid = torch.empty(nz, ny + 2 * r, X, device="cuda").uniform_(
+        -1, 1, generator=torch.Generator(device="cuda").manual_seed(r))
+    even = X + (2 - X) % 4
+    for base, py in ((1, X), (0, X | 1), (2, even), (0, even)):
+        inp = unaligned(grid, base, py)
+        mms.apply(shape, r, c, inp)
+        assert mms.last_planes() == 8
+        assert same_as_naive(shape, r, c, inp), (base, py)
