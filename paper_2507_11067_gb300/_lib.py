@@ -43,7 +43,7 @@ NOALLOC_MAX_POINTS = 8388608  # MMS_NOALLOC_MAX_POINTS of include/mms.h
 EXPORTS = ["mms_stencil_apply", "mms_stencil_apply_ex", "mms_auto_path", "mms_num_variants",
            "mms_default_variant",
            "mms_set_variant", "mms_wave_step", "mms_wave_forward", "mms_wave_adjoint",
-           "mms_model_from_velocity", "mms_grad_to_velocity", "mms_dot_f64", "mms_last_error",
+           "mms_model_from_velocity", "mms_grad_to_velocity", "mms_dot_f64", "mms_last_error", "mms_last_planes",
            "mms_check_device", "mms_version", "mms_stencil_apply_noalloc", "mms_wave_step_to",
            "mms_sum_f64", "mms_selftest_timeout", "mms_stencil_apply_host", "mms_vti_model", "mms_vti_step",
            "mms_aniso_num_variants", "mms_aniso_set_variant", "mms_tti_model", "mms_tti_step", "mms_stencil_apply_f64", "mms_wave_step_lap",
