@@ -684,11 +684,14 @@ __global__ void __launch_bounds__(kRowThreads *kRowsPerBlock)
 // of mu^{n+1} (L a^n) turned into dJ/dm.  GB300's FP64 pipe makes an IEEE
 // division per point the whole cost (256^3: 635 us, HBM's time is 49), so the
 // quotient comes from a reciprocal of the FP32 m, kept as the sum of two FP32
-// values (r + e, 48 bits, worked out on the FP32 pipe), and one FP64
-// correction step: q = g r', q += (g - q m) r', within an ulp of the
-// quotient.  What that cannot serve (m outside 2^-60 .. 2^60, a quotient that
-// is no number of moderate size) divides; the range is read off the bits, on
-// the integer pipe.
+// values (r + e, 47 bits, worked out on the FP32 pipe), and one FP64
+// correction step: q = g r', q += (g - q m) r'.  That is the IEEE quotient: the
+// first q is within 70 ulps, so g - q m (at most 32 bits) is exact, and the sum
+// before its rounding is within 2^-40 ulp of g / m -- while a quotient of a
+// 53-bit by a 24-bit number is at least 2^-25 ulp from every midpoint, so both
+// round alike.  What this cannot serve (m outside 2^-60 .. 2^60, a quotient
+// that is no number of moderate size) divides; the range is read off the bits,
+// on the integer pipe.
 __device__ __forceinline__ double divide_by_float(double g, float m)
 {
     if (m >= 0x1p-60f && m <= 0x1p60f) {
