@@ -186,8 +186,7 @@ struct Cfg {
     // Output subtiles staged for TMA stores (one TXO x TY box per epilogue
     // warp and output, two buffers per warp); a subtile row is a 16-byte
     // multiple (TXO % 4 == 0).
-    static constexpr bool TSTORE = (TXO * 4) % 16 == 0;
-    static constexpr int OBUF = TSTORE ? (TXO * TY * 4 + 127) / 128 * 128 : 0;
+    static constexpr int OBUF = (TXO * TY * 4 + 127) / 128 * 128;
     static constexpr size_t OFF_OBUF = OFF_BAR + 1024;
     static constexpr size_t SMEM_NEED = 1024 + OFF_OBUF + 8 * NEPI * (size_t)OBUF;
     // a single CTA takes at least 120 KB, so that two CTAs holding all 512
@@ -197,6 +196,7 @@ struct Cfg {
     static_assert(OK, "tensor-core configuration does not fit");
     static constexpr uint32_t IDESC = tc::instr_desc(BF ? 1u : 2u, 128, N);
     static_assert(BOXW >= TX - TXO + K && BOXW % 4 == 0 && (BOXW / 4) % 2 == 1, "staging box");
+    static_assert(TXO % 4 == 0, "subtile rows are 16-byte multiples");
     static_assert(N % 16 == 0 && N <= 256 && (N == 48 || N == 64 || N == 80), "epilogue loads");
     static_assert(2 * NST + 2 * PR + 2 * ND <= 120, "barrier area");
     // TMEM operand and accumulator columns start on 16-column boundaries
@@ -554,18 +554,10 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
             // the 16 input values of this lane's row
             float v[16];
             const float *row = stg + (size_t)st * (C::STG_STRIDE / 4) + t * C::BOXW + q * C::TXO;
-            if constexpr (C::TXO % 4 == 0) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float4 f = reinterpret_cast<const float4 *>(row)[i];
-                    v[4 * i] = f.x; v[4 * i + 1] = f.y; v[4 * i + 2] = f.z; v[4 * i + 3] = f.w;
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float2 f = reinterpret_cast<const float2 *>(row)[i];
-                    v[2 * i] = f.x; v[2 * i + 1] = f.y;
-                }
+            for (int i = 0; i < 4; ++i) {
+                const float4 f = reinterpret_cast<const float4 *>(row)[i];
+                v[4 * i] = f.x; v[4 * i + 1] = f.y; v[4 * i + 2] = f.z; v[4 * i + 3] = f.w;
             }
             const uint32_t acol = lane_base + (uint32_t)(C::A0 + as * C::APL);
             if constexpr (C::BF) {
@@ -693,31 +685,29 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
                 o[x] = acc;
             }
             const int xb = x0 + q * C::TXO, zg = z0 + z;
-            if constexpr (C::TSTORE) {
-                if (a.tstore) {
-                    // the subtile into this warp's buffer for the output's
-                    // parity, then one TMA store (clipped at the grid's edges);
-                    // the store that last read the buffer is waited for first
-                    float *ob = obuf + (size_t)(nout & 1) * (C::OBUF / 4);
-                    if (lane == 0) bulk_wait_read_all();
-                    __syncwarp();
-                    if (t < C::TY) {
+            if (a.tstore) {
+                // the subtile into this warp's buffer for the output's
+                // parity, then one TMA store (clipped at the grid's edges);
+                // the store that last read the buffer is waited for first
+                float *ob = obuf + (size_t)(nout & 1) * (C::OBUF / 4);
+                if (lane == 0) bulk_wait_read_all();
+                __syncwarp();
+                if (t < C::TY) {
 #pragma unroll
-                        for (int i = 0; i < C::TXO / 4; ++i)
-                            reinterpret_cast<float4 *>(ob + t * C::TXO)[i] =
-                                make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
-                    }
-                    ptx::fence_proxy_async_smem();  // generic writes -> the TMA unit's reads
-                    __syncwarp();
-                    if (lane == 0 && xb < a.nx) {
-                        tma_store_3d(&omap, ob, xb, y0, zg);
-                        bulk_commit();
-                    }
-                    ++nout;
-                    if (lane == 0 && q == 0) MMS_TL(8, j);
-                    tep += MMS_CLOCK() - t1;
-                    return true;
+                    for (int i = 0; i < C::TXO / 4; ++i)
+                        reinterpret_cast<float4 *>(ob + t * C::TXO)[i] =
+                            make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
                 }
+                ptx::fence_proxy_async_smem();  // generic writes -> the TMA unit's reads
+                __syncwarp();
+                if (lane == 0 && xb < a.nx) {
+                    tma_store_3d(&omap, ob, xb, y0, zg);
+                    bulk_commit();
+                }
+                ++nout;
+                if (lane == 0 && q == 0) MMS_TL(8, j);
+                tep += MMS_CLOCK() - t1;
+                return true;
             }
             if constexpr (MODE == M_STAR) {
                 // from registers: the star's epilogue has none left for the form
@@ -726,7 +716,7 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
                 if (t < C::TY && y < a.ny && xb < a.nx) {
                     float *op = a.out + (int64_t)zg * a.opz + (int64_t)y * a.opy + xb;
                     const bool full = xb + C::TXO <= a.nx;
-                    if (C::TXO % 4 == 0 && full && a.vec == 4) {
+                    if (full && a.vec == 4) {
 #pragma unroll
                         for (int i = 0; i < C::TXO / 4; ++i)
                             reinterpret_cast<float4 *>(op)[i] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
@@ -822,8 +812,7 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
                     out_fix();
                 }
             }
-            if constexpr (C::TSTORE)
-                if (lane == 0) bulk_wait_all();
+            if (lane == 0) bulk_wait_all();
         } else if (wi == 0) {
             // every staged plane in order (the star's z sums in registers)
             float zq[MODE == M_STAR ? W : 1][MODE == M_STAR ? C::TXO : 1];
@@ -851,8 +840,7 @@ __global__ void __launch_bounds__(Cfg<R, PREC, MODE>::NT, Cfg<R, PREC, MODE>::DU
             }
             // this warp's output stores are complete (and their sources
             // read) before the CTA exits
-            if constexpr (C::TSTORE)
-                if (lane == 0) bulk_wait_all();
+            if (lane == 0) bulk_wait_all();
         }
         if (!ok) *abort_flag = 1;
         if (lane == 0 && warp == 4) {
@@ -952,7 +940,7 @@ cudaError_t launch_r(const Sweep &s, const CUtensorMap &map, int nzt, const Laun
     const uintptr_t ob = reinterpret_cast<uintptr_t>(L.out);
     a.vec = (L.opy % 4 == 0 && L.opz % 4 == 0 && ob % 16 == 0) ? 4 : (L.opy % 2 == 0 && L.opz % 2 == 0 && ob % 8 == 0) ? 2 : 1;
     a.tstore = a.vec == 4 &&
-               encode_tmap_3d(&omap, L.out, s.nx, s.ny, s.nz, L.opy, L.opz, C::TSTORE ? C::TXO : 4, C::TY, 1);
+               encode_tmap_3d(&omap, L.out, s.nx, s.ny, s.nz, L.opy, L.opz, C::TXO, C::TY, 1);
     const int slots = sl.sms * sl.per_sm;
     const int grid = a.tiles < slots ? a.tiles : slots;
     kern<<<grid, C::NT, C::SMEM, s.stream>>>(map, omap, cf, a, device_error_word());
