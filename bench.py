@@ -68,14 +68,27 @@ WORKLOAD_NAMES = {
 }
 WORKLOAD_NAMES["fp64_512"] = ("FP64 sweeps: star r=4 (FD8 weights) and box r=1 (weights N(0, 1/27)), 512^3 "
                               "FP64 interior + halo, input U[-1, 1]")
-ANISO = {"vti512": dict(kind="vti", n=512, shots=4, bytes_per_point_step=32,
+ANISO = {"vti512": dict(kind="vti", n=512, shots=4,
                         kernel="vti_fwd_kernel (two coupled r=4 stars + leapfrog + sponge + source + receivers)"),
-         # per point-step: the p pass (read p and the tilt, 16 B; write Lap p
-         # and H1 p, 8 B) and the q pass with the combine fused in (read q,
-         # Lap p, H1 p, the 8 medium fields, p^n, p^{n-1}, q^{n-1}: 56 B;
-         # write p^{n+1}, q^{n+1}: 8 B)
-         "tti512": dict(kind="tti", n=512, shots=2, bytes_per_point_step=88,
+         "tti512": dict(kind="tti", n=512, shots=2,
                         kernel="whole step: tti_deriv_kernel<p> + tti_deriv_kernel<q, combine fused>")}
+
+
+def step_bytes(kind: str, shots: int) -> float:
+    """Algorithmic bytes per shot-point of one step: the shots' own fields read
+    and written once, the medium once for all of them (the shots of a tile run
+    next to each other and read it from L2).
+    rtm: a^n, a^{n-1} in, a^{n+1} out; m shared.
+    grad: that; the recompute step with L a^n out as well; the adjoint step (its
+    state at n+1, n+2 and L a^n in, the state at n out); m shared in each, and
+    the FP64 gradient's read and write (16 B) once for all shots.
+    vti: two fields at n, n-1 in and at n+1 out; two medium fields shared.
+    tti: the p pass (p in; Lap p, H1 p out; three tilt fields shared) and the q
+    pass (q, Lap p, H1 p, p^n, p^{n-1}, q^{n-1} in; p^{n+1}, q^{n+1} out; eight
+    medium fields shared)."""
+    own, shared = {"rtm": (12, 4), "grad": (12 + 16 + 16, 3 * 4 + 16), "vti": (24, 8),
+                   "tti": (12 + 32, 12 + 32)}[kind]
+    return own + shared / shots
 
 
 def sweep_coeffs(shape, r):
@@ -792,7 +805,8 @@ def run_wave(args):
     pts = nshots * n ** 3
     if args.workload == "rtm512":
         units = world * pts * steps
-        bytes_alg = 16.0 * pts * steps
+        bpp = step_bytes("rtm", nshots)
+        bytes_alg = bpp * pts * steps
         # end to end: velocity and wavelet in from pinned host memory, records out
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record(stream)
@@ -814,9 +828,9 @@ def run_wave(args):
                 "frac": bytes_alg / elapsed / 1e9 / hbm_peak,
                 "traffic": captured_traffic("wave_fwd r=4", pts),
                 "kernel": "wave_fwd_kernel (fused star r=4 + leapfrog + sponge + source + receivers)",
-                "bytes_per_point_step": 16}
+                "bytes_per_point_step": bpp}
         if roof["traffic"]:
-            roof["traffic_over_algorithmic"] = roof["traffic"] / (16.0 * pts)
+            roof["traffic_over_algorithmic"] = roof["traffic"] / (bpp * pts)
         unit = "GPoint-steps/s"
     else:
         units = world * pts * nsteps * steps
@@ -841,12 +855,7 @@ def run_wave(args):
         e2e = {"value": job_rate(world, pts * nsteps, e2e_s), "unit": "GPoint-steps/s (forward + gradient)",
                "h2d_bytes_per_step": v0_host.numel() * 4 + amps_host.numel() * 4 + obs_host.numel() * 4,
                "d2h_bytes_per_step": g_host.numel() * g_host.element_size()}
-        # per shot-point and step: forward 16 B, recompute 20 B (out of place,
-        # no copies; it also writes L a^n), adjoint 20 B (its state at n+1
-        # and n+2, m, L a^n read, the state at n written), and the FP64
-        # gradient's read-modify-write, 16 B per point shared by the shots
-        # (their reductions meet in L2)
-        bpp = 56.0 + 16.0 / nshots
+        bpp = step_bytes("grad", nshots)
         bytes_alg = bpp * pts * nsteps * steps
         ri = prop.r
         mu = args.adjoint == "mu" or (args.adjoint == "auto" and bool((prop.m[ri:-ri, ri:-ri, ri:-ri] > 0).all()))
@@ -957,7 +966,7 @@ def run_aniso(args):
     clk = clocks.stop()
     elapsed = max_over_ranks(t0.elapsed_time(t1) / 1e3, dist, dev)
     pts = nshots * n ** 3
-    bpp = spec["bytes_per_point_step"]
+    bpp = step_bytes(spec["kind"], nshots)
     bytes_alg = float(bpp) * pts * steps
     # end to end: the medium and the wavelet in from pinned host memory, the
     # model kernel, the steps with receivers, the records out
@@ -1092,7 +1101,7 @@ def run_f64(args):
     flops = 2 * fmas[shape](r) * n ** 3
     roof = {"bound": "alu", "achieved": flops / (kms[di] / 1e3) / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",
             "frac": flops / (kms[di] / 1e3) / 1e12 / fp64_peak, "traffic": captured_traffic(f"f64 {shape} r={r}", n ** 3),
-            "kernel": f"f64_kernel {shape} r={r} {n}^3", "ms": kms[di],
+            "kernel": f"{'f64_star_kernel' if shape == 'star' else 'f64_kernel'} {shape} r={r} {n}^3", "ms": kms[di],
             "peak_note": f"{n_sm} SMs x 2 FP64 FMA/clock x 2 flop x {sm_max_mhz:.0f} MHz (GB300's nominal FP64 rate)",
             "flop_per_point": 2 * fmas[shape](r)}
     sweeps = {f"{sh} r={rr}": {"ms": kms[i], "gpts": n_ ** 3 / (kms[i] / 1e3) / 1e9,
@@ -1190,8 +1199,7 @@ def _roof_entry(ms_step, pts, bpp, hbm_peak, err, config):
 
 def extra_rtm(mms, torch, dev, hbm_peak, steps=20):
     """The acoustic forward workload in brief: 8 shots x 512^3, `steps`
-    graph-launched steps (read a^n, a^{n-1}; write a^{n+1}: 16 B per
-    point-step with m shared by the shots), from seeded random states; then
+    graph-launched steps, from seeded random states; then
     one more step, checked at sampled points of shot 0."""
     import oracle
     from paper_2507_11067_gb300.wave import WavePropagator
@@ -1217,7 +1225,7 @@ def extra_rtm(mms, torch, dev, hbm_peak, steps=20):
                                   cur, prev, pts)
     idx = torch.from_numpy(pts).to(dev)
     got = nxt[0][idx[:, 2] + R, idx[:, 1] + R, idx[:, 0] + R].double().cpu().numpy()
-    return _roof_entry(ms, ns * n ** 3, 16, hbm_peak, rel_err(got, ref),
+    return _roof_entry(ms, ns * n ** 3, step_bytes("rtm", ns), hbm_peak, rel_err(got, ref),
                        f"{ns} shots x {n}^3, {steps} steps in one CUDA graph, from seeded random states")
 
 
@@ -1244,7 +1252,7 @@ def extra_grad(mms, torch, dev, hbm_peak):
 
     ms = _time(gradient, reps=2)
     pts = ns * n ** 3
-    bpp = 56.0 + 16.0 / ns
+    bpp = step_bytes("grad", ns)
     f = [prop.new_fields() for _ in range(5)]
     _fill_interior(f, R, torch.Generator(device=dev).manual_seed(50))
     resid = torch.randn((ns, n, n), device=dev, generator=torch.Generator(device=dev).manual_seed(51))
@@ -1295,8 +1303,8 @@ def extra_grad(mms, torch, dev, hbm_peak):
             "forward_step_us": 1e3 * t_fwd, "recompute_step_us": 1e3 * t_rec, "adjoint_step_us": 1e3 * t_adj,
             "adjoint_lam_step_us": 1e3 * t_adj_lam, "adjoint": prop.adjoint,
             "max_rel_err": max(errs),
-            "config": f"{ns} shots x {n}^3, {nsteps} steps, checkpoint every {every}; byte model: forward 16, "
-                      f"recompute 20, adjoint 20 B per shot-point-step + FP64 gradient 16 B per point-step"}
+            "config": f"{ns} shots x {n}^3, {nsteps} steps, checkpoint every {every}; byte model per point-step: "
+                      "forward 12, recompute 16, adjoint 16 B per shot, m 12 B and the FP64 gradient 16 B shared"}
 
 
 def _aniso_setup(mms, torch, dev, kind, n, ns, steps):
@@ -1311,7 +1319,7 @@ def _aniso_setup(mms, torch, dev, kind, n, ns, steps):
 
 def extra_vti(mms, torch, dev, hbm_peak, steps=10):
     """The VTI workload in brief: 4 shots x 512^3, `steps` fused steps from
-    seeded random states (32 B per point-step); one more step checked at
+    seeded random states; one more step checked at
     sampled points of shot 0."""
     from oracle import aniso
     n, ns, r = 512, 4, 4
@@ -1341,13 +1349,13 @@ def extra_vti(mms, torch, dev, hbm_peak, steps=10):
     idx = torch.from_numpy(pts).to(dev)
     got = [t[0][idx[:, 2] + r, idx[:, 1] + r, idx[:, 0] + r].double().cpu().numpy() for t in (f[4], f[5])]
     err = max(rel_err(got[0], oh), rel_err(got[1], ov))
-    return _roof_entry(ms, ns * n ** 3, ANISO["vti512"]["bytes_per_point_step"], hbm_peak, err,
+    return _roof_entry(ms, ns * n ** 3, step_bytes("vti", ns), hbm_peak, err,
                        f"{ns} shots x {n}^3, {steps} steps from seeded random states")
 
 
 def extra_tti(mms, torch, dev, hbm_peak, steps=10):
     """The TTI workload in brief: 2 shots x 512^3, `steps` steps (two launches
-    each; 88 B per point-step) from seeded random states; one more step
+    each) from seeded random states; one more step
     checked at sampled points of shot 0."""
     from oracle import aniso
     n, ns, r = 512, 2, 4
@@ -1381,7 +1389,7 @@ def extra_tti(mms, torch, dev, hbm_peak, steps=10):
     idx = torch.from_numpy(pts).to(dev)
     got = [t[0][idx[:, 2] + r, idx[:, 1] + r, idx[:, 0] + r].double().cpu().numpy() for t in (f[4], f[5])]
     err = max(rel_err(got[0], op), rel_err(got[1], oq))
-    return _roof_entry(ms, ns * n ** 3, ANISO["tti512"]["bytes_per_point_step"], hbm_peak, err,
+    return _roof_entry(ms, ns * n ** 3, step_bytes("tti", ns), hbm_peak, err,
                        f"{ns} shots x {n}^3, {steps} steps from seeded random states")
 
 
