@@ -206,15 +206,16 @@ def bf16_sustained_peak():
     return 1700.0, "fallback sustained"
 
 
-def captured_traffic(key: str, points: int):
+def captured_traffic(key: str, points: int, shots: int | None = None):
     """DRAM bytes of one launch from the committed ncu capture of this kernel
     (profiles/traffic.json), scaled by points; None when the kernel's sources
-    changed since the capture."""
+    changed since the capture, or where it ran another number of shots (they
+    share the medium, so the bytes per shot-point depend on it)."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
         return None
     rec = json.load(open(p)).get(key)
-    if not rec:
+    if not rec or rec.get("shots") != shots:
         return None
     for f, h in rec["sources"].items():
         path = os.path.join(ROOT, "paper_2507_11067_gb300", "csrc", f)
@@ -826,7 +827,7 @@ def run_wave(args):
                "h2d_bytes_per_step": h2d / steps, "d2h_bytes_per_step": d2h / steps}
         roof = {"bound": "hbm", "achieved": bytes_alg / elapsed / 1e9, "peak": hbm_peak, "unit": "GB/s",
                 "frac": bytes_alg / elapsed / 1e9 / hbm_peak,
-                "traffic": captured_traffic("wave_fwd r=4", pts),
+                "traffic": captured_traffic("wave_fwd r=4", pts, nshots),
                 "kernel": "wave_fwd_kernel (fused star r=4 + leapfrog + sponge + source + receivers)",
                 "bytes_per_point_step": bpp}
         if roof["traffic"]:
@@ -988,7 +989,7 @@ def run_aniso(args):
            "h2d_bytes_per_step": h2d / steps, "d2h_bytes_per_step": d2h / steps}
     key = f"{spec['kind']}_fwd r=4"
     roof = {"bound": "hbm", "achieved": bytes_alg / elapsed / 1e9, "peak": hbm_peak, "unit": "GB/s",
-            "frac": bytes_alg / elapsed / 1e9 / hbm_peak, "traffic": captured_traffic(key, nshots * n ** 3),
+            "frac": bytes_alg / elapsed / 1e9 / hbm_peak, "traffic": captured_traffic(key, nshots * n ** 3, nshots),
             "kernel": spec["kernel"], "bytes_per_point_step": bpp}
     if roof["traffic"]:
         roof["traffic_over_algorithmic"] = roof["traffic"] / (float(bpp) * pts)
