@@ -121,8 +121,10 @@ typedef struct {
  * variant.  The TMA-staged paths need in_pitch_y*4 and in_pitch_z*4 to be
  * multiples of 16 bytes and `in` 16-byte aligned; with MMS_PATH_AUTO an
  * input that breaks this runs on the CUDA cores with plain copies of its
- * planes instead of TMA (FP32, any pitch), with a forced TMA path it
- * returns MMS_E_ALIGN.  Tensor-core paths support the box and the star of
+ * planes instead of TMA (FP32; point by point where in_pitch_y is 2^24 floats
+ * or more, the input is not 4-byte aligned, or a planar grid has more than
+ * 65535 planes or 65535 x 32 rows), with a forced TMA path it returns
+ * MMS_E_ALIGN.  Tensor-core paths support the box and the star of
  * radius 1..4.  The star's variants come in two forms.  The first half
  * (the library's choice) sweep it in one pass: the in-plane x/y part as
  * banded tensor-core products, the 2r z terms as FP32 multiply-adds on the
@@ -168,8 +170,8 @@ mms_status mms_stencil_apply_host(const mms_stencil_desc *desc, const float *hos
  * measured best variant, and it holds a BF16x3 row only where that path beat
  * the CUDA cores.  Elsewhere AUTO takes the TMA CUDA-core path.  For unaligned
  * input the answer is MMS_PATH_NAIVE, the path for any pitch (AUTO stages the
- * planes by plain copies there; MMS_PATH_NAIVE itself, forced, reads point by
- * point).  Host only; the first call on a device reads
+ * planes by plain copies there where they fit, see mms_stencil_apply_ex;
+ * MMS_PATH_NAIVE itself, forced, reads point by point).  Host only; the first call on a device reads
  * the device's name (cudaGetDeviceProperties). */
 int32_t mms_auto_path(int shape, int radius, int tma_aligned);
 

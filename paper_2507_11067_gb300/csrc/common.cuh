@@ -158,7 +158,12 @@ cudaError_t kernel_slots(SlotCache &cache, const void *kern, int threads, size_t
 // 172 us, 196 us in finer ones).  Otherwise the chunk is the one of least
 // modelled time among those that fill one wave to 1, 2, ... CTAs per SM or run
 // in one and a half to four waves: the VTI step on 2 x 250 x 230 x 190, 232
-// columns on 456 CTA slots, takes 285 us as one chunk each, 174 us in five.
+// columns on 456 CTA slots, takes 285 us as one chunk each, 171 us in five.
+// Against the tuned chunk everywhere, over 36 random shapes per kernel (mean
+// and worst time, kernels that changed in nothing else): star r = 1 0.54, 1.04;
+// r = 2 0.53, 1.01; box r = 1 0.45, 1.04; r = 2 0.57, 1.00; planar star r = 2
+// 0.88, 1.00; planar box r = 3 0.91, 1.00.  VTI and TTI, their paired updates
+// included: 0.42, 0.98 and 0.64, 0.98.
 int z_chunk(const Slots &sl, int64_t cols, int64_t nz, int halo, int tz, int threads);
 
 // How a kernel's CTAs divide the columns they march along z: CTA b marches

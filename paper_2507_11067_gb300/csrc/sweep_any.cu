@@ -11,9 +11,12 @@
 // the tile's padding and the columns and rows past the grid are not read, and
 // feed no stored output.
 //
-// Bound by HBM where the one-thread-per-point kernel was bound by its loads
-// (6r + 1 or (2r+1)^3 of them per point): star r = 2 on 301 x 260 x 230, 166
-// -> 43 us (3.4 TB/s); box r = 1 on a dense 512^3, 2.87 -> 0.22 ms.
+// The one-thread-per-point kernel was bound by its loads (6r + 1 or (2r+1)^3 of
+// them per point): star r = 2 on 301 x 260 x 230, 166 -> 43 us (3.4 TB/s of
+// algorithmic bytes, half of HBM's rate); box r = 1 on a dense 512^3, 2.87 ->
+// 0.22 ms.  What binds now is the copies: eleven of 4 bytes per thread and
+// plane, whose instructions fill the load/store queue (star r = 2 on a dense
+// 511 x 512 x 512: issue 47 %, DRAM 52 %, mio_throttle the top stall).
 #include "common.cuh"
 #include "tile.cuh"
 

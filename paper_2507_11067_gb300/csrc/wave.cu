@@ -3,9 +3,10 @@
 //
 // The forward kernel is the star sweep of sweep_cc.cu with the leapfrog
 // update fused into its epilogue: the Laplacian of a^n never leaves
-// registers, so one step moves 16 bytes per point (read a^n, a^{n-1}, m;
-// write a^{n+1}) plus the L2-served halos.  Shots are independent and run
-// as separate grid slices of the same launch.
+// registers, so one step moves 12 bytes per point and shot (read a^n, a^{n-1};
+// write a^{n+1}) and 4 of m for all of them, plus the L2-served halos.  Shots
+// are independent; those of a tile are neighbours in launch order, so that they
+// share m in L2.
 //
 // The adjoint kernel computes, per point and shot,
 //   lam^n = R^T r^n + 2 g lam^{n+1} + L(m g lam^{n+1}) - g^2 lam^{n+2}
