@@ -324,7 +324,9 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, PY, S>::NT)
                     // other: a few roundings near the source decide the error
                     // of a whole run.  With fma(m, L a, 2 a) in the middle the
                     // gradient's error of 2 shots on 256^3, 40 steps, was
-                    // 1.3e-6 where this has 5.4e-7, at the same speed.
+                    // 1.3e-6 where this has 5.4e-7.  (16 steps of 8 x 512^3
+                    // take 42.08 ms, 41.77 with that; an add of 2 a to the
+                    // product compiles into that fma again.)
                     const f2 t = mul2(pair(mv[i][2 * h], mv[i][2 * h + 1]), acc[0][i][h]);
                     const f2 u = fma2(pair(2.f, 2.f), c, t);
                     unpair(gg, g[2 * h], g[2 * h + 1]);
