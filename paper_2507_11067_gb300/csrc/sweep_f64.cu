@@ -18,22 +18,23 @@ struct F64Star {
     double c[kMaxStar], centre;
 };
 
-// The star: a thread computes ZP points of one z column, so that their z
-// neighbours are loaded once ((ZP + 2R) / ZP loads per point along z instead
-// of 2R + 1).  Bound by the FP64 pipe, which does nothing but the 6R + 1 FMAs
-// of a point: the centre weight is folded on the host (two FP64 adds per point
-// before, 256^3 r = 4: 864 -> 802 us), and the weights sit in registers, for
-// FMAs with a constant-bank operand run at five sixths of the pipe's rate
-// whatever the tile (802 -> 717 us; the pipe's 25 FMAs take 667).  Small CTAs
-// spread evenly (four rows: 734 us).
-constexpr int kStarZP = 4, kStarBY = 2;
+// The star, one point per thread.  Bound by the FP64 pipe, which does nothing
+// but the 6R + 1 FMAs of a point: the centre weight is folded on the host (two
+// FP64 adds per point before, 256^3 r = 4: 864 -> 802 us), and the weights sit
+// in registers, for FMAs with a constant-bank operand run at five sixths of the
+// pipe's rate whatever the tile (802 -> 698 us; the pipe's 25 FMAs take 667).
+// Small CTAs spread evenly, and with one point per thread small grids fill the
+// SMs (four points of a z column per thread, their z neighbours loaded once:
+// r = 4, 256^3 715 us, 31 x 33 x 35 5.5 against 3.7, r = 3, 129 x 33 x 65 20.9
+// against 13.7).
+constexpr int kStarBY = 2;
 
 template <int R>
 __global__ void __launch_bounds__(32 * kStarBY)
     f64_star_kernel(const __grid_constant__ F64Star cf, const double *__restrict__ in, int64_t ipy, int64_t ipz,
                     double *__restrict__ out, int64_t opy, int64_t opz, int nx, int ny, int nz)
 {
-    constexpr int W = 2 * R + 1, ZP = kStarZP;
+    constexpr int W = 2 * R + 1;
     // by way of shared memory, or the compiler takes them from the constant bank
     __shared__ double sw[3 * W + 1];
     for (int i = threadIdx.y * 32 + threadIdx.x; i <= 3 * W; i += 32 * kStarBY) sw[i] = i < 3 * W ? cf.c[i] : cf.centre;
@@ -45,33 +46,20 @@ __global__ void __launch_bounds__(32 * kStarBY)
     const int x = blockIdx.x * 32 + threadIdx.x;
     if (x >= nx) return;
     // y and z stride over the grid's extents (launch dims are capped at 65535)
-    for (int z = blockIdx.z * ZP; z < nz; z += gridDim.z * ZP)
+    for (int z = blockIdx.z; z < nz; z += gridDim.z)
         for (int y = blockIdx.y * kStarBY + threadIdx.y; y < ny; y += gridDim.y * kStarBY) {
-            const double *c0 = in + (int64_t)(z + R) * ipz + (int64_t)(y + R) * ipy + (x + R);
-            const int n = min(ZP, nz - z);  // points of this column inside the grid
-            double col[ZP + 2 * R];         // planes z - R .. z + ZP - 1 + R
+            const double *c = in + (int64_t)(z + R) * ipz + (int64_t)(y + R) * ipy + (x + R);
+            double a = centre * __ldg(c);
 #pragma unroll
-            for (int i = 0; i < ZP + 2 * R; ++i) col[i] = i < n + 2 * R ? __ldg(c0 + (i - R) * ipz) : 0.0;
-            double acc[ZP];
-#pragma unroll
-            for (int i = 0; i < ZP; ++i) {
-                if (i >= n) break;
-                const double *c = c0 + i * ipz;
-                double a = centre * col[i + R];
-#pragma unroll
-                for (int d = 1; d <= R; ++d) {
-                    a = fma(w[R + d], __ldg(c + d), a);
-                    a = fma(w[R - d], __ldg(c - d), a);
-                    a = fma(w[W + R + d], __ldg(c + d * ipy), a);
-                    a = fma(w[W + R - d], __ldg(c - d * ipy), a);
-                    a = fma(w[2 * W + R + d], col[i + R + d], a);
-                    a = fma(w[2 * W + R - d], col[i + R - d], a);
-                }
-                acc[i] = a;
+            for (int d = 1; d <= R; ++d) {
+                a = fma(w[R + d], __ldg(c + d), a);
+                a = fma(w[R - d], __ldg(c - d), a);
+                a = fma(w[W + R + d], __ldg(c + d * ipy), a);
+                a = fma(w[W + R - d], __ldg(c - d * ipy), a);
+                a = fma(w[2 * W + R + d], __ldg(c + d * ipz), a);
+                a = fma(w[2 * W + R - d], __ldg(c - d * ipz), a);
             }
-#pragma unroll
-            for (int i = 0; i < ZP; ++i)
-                if (i < n) out[(int64_t)(z + i) * opz + (int64_t)y * opy + x] = acc[i];
+            out[(int64_t)z * opz + (int64_t)y * opy + x] = a;
         }
 }
 
@@ -126,7 +114,7 @@ cudaError_t f64_star(int r, const double *w, const double *in, int64_t ipy, int6
     const int W = 2 * r + 1;
     for (int i = 0; i < 3 * W; ++i) cf.c[i] = w[i];
     cf.centre = w[r] + w[W + r] + w[2 * W + r];
-    const dim3 block(32, kStarBY), grid((nx + 31) / 32, min((ny + kStarBY - 1) / kStarBY, 65535), min((nz + kStarZP - 1) / kStarZP, 65535));
+    const dim3 block(32, kStarBY), grid((nx + 31) / 32, min((ny + kStarBY - 1) / kStarBY, 65535), min(nz, 65535));
     switch (r) {
         case 1: f64_star_kernel<1><<<grid, block, 0, st>>>(cf, in, ipy, ipz, out, opy, opz, nx, ny, nz); break;
         case 2: f64_star_kernel<2><<<grid, block, 0, st>>>(cf, in, ipy, ipz, out, opy, opz, nx, ny, nz); break;
