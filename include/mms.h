@@ -121,7 +121,9 @@ typedef struct {
  * variant.  The TMA-staged paths need in_pitch_y*4 and in_pitch_z*4 to be
  * multiples of 16 bytes and `in` 16-byte aligned; with MMS_PATH_AUTO an
  * input that breaks this runs on the CUDA cores with plain copies of its
- * planes instead of TMA (FP32; point by point where in_pitch_y is 2^24 floats
+ * planes instead of TMA (FP32; point by point on small grids, where that is
+ * faster -- stars of fewer than 300000 points, boxes of radius 4 of fewer than
+ * 100000, planar stars of fewer than 4096 -- and where in_pitch_y is 2^24 floats
  * or more, the input is not 4-byte aligned, or a planar grid has more than
  * 65535 planes or 65535 x 32 rows), with a forced TMA path it returns
  * MMS_E_ALIGN.  Tensor-core paths support the box and the star of

@@ -269,11 +269,29 @@ cudaError_t launch_r(const Sweep &s)
 
 }  // namespace
 
+// Points from which the staged kernels are the faster ones.  Below, a march's
+// latency (its planes one after the other) is longer than the point-by-point
+// kernel's single chain of loads.  Device time, point by point against staged:
+// star r = 4, 9^3 3.0 and 4.7 us, 57^3 5.0 and 5.6, 65 x 67 x 63 (274 k points)
+// 6.1 and 7.0, 129 x 33 x 65 6.2 and 7.4; 255 x 255 x 5 (325 k) and 95^3 the
+// other way round, 79^3 8.1 and 8.9 at r = 3, at r = 1 even from 41^3 on; box r =
+// 4, 31^3 38 and 42 us, 15 x 20 x 301 46 and 57, 47^3 the other way round (boxes
+// of smaller radius at every size); planar star 17^2 2.0 and 2.2, 65^2 even.
+static int64_t staged_from(int shape, int r)
+{
+    switch (shape) {
+        case MMS_STAR: return 300000;
+        case MMS_BOX: return r == 4 ? 100000 : 0;
+        case MMS_STAR2D: return 4096;
+        default: return 0;
+    }
+}
+
 // Row offsets inside a staged tile (at most 40 rows) are 32-bit, input
 // elements 4-byte aligned, and the planar grid's launch extents are CUDA's.
 bool any_pitch_ok(const Sweep &s)
 {
-    return s.ipy < (1 << 24) && reinterpret_cast<uintptr_t>(s.in) % 4 == 0 &&
+    return s.nx * s.ny * s.nz >= staged_from(s.shape, s.r) && s.ipy < (1 << 24) && reinterpret_cast<uintptr_t>(s.in) % 4 == 0 &&
            (!is_planar(s.shape) || (s.nz <= 65535 && s.ny <= (int64_t)65535 * 32));
 }
 
