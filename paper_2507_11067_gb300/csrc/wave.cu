@@ -649,29 +649,41 @@ __global__ void __launch_bounds__(Geom<R, TX, TY, 1, S>::NT, 2)
         if (!plane(j)) return;
 }
 
-// The pointwise kernels below run over rows of x (blocks of 4 rows, 64 threads
-// along each), so that a point's place costs no division: with one per
-// coordinate and point they took four times HBM's time (256^3: model 94 -> 26
-// us).
-constexpr int kRowThreads = 64, kRowsPerBlock = 4;
-inline int row_blocks(int64_t rows)
+// The pointwise kernels below run over rows of x, so that a point's place costs
+// no division: with one per coordinate and point they took four times HBM's
+// time (256^3: model 94 -> 26 us).  A block is 256 threads, 64 along each of
+// four rows; narrow grids take fewer along more rows (5 x 300 x 300: model 17.5
+// -> 7.4 us, division 25 -> 8.2).  T, the threads along x, is a template
+// argument: with it in blockDim the loop along x is not unrolled (256^3: model
+// 28 -> 45 us).
+constexpr int kRowThreads = 256;
+template <typename F>
+void launch_rows(int64_t X, int64_t rows, F launch)
 {
-    const int64_t b = (rows + kRowsPerBlock - 1) / kRowsPerBlock;
-    return (int)(b < 152 * 32 ? b : 152 * 32);
+    const auto go = [&](auto t) {
+        constexpr int T = decltype(t)::value, per = kRowThreads / T;
+        const int64_t b = (rows + per - 1) / per;
+        launch(t, (int)(b < 152 * 32 ? b : 152 * 32), dim3(T, per));
+    };
+    if (X <= 8) go(std::integral_constant<int, 8>{});
+    else if (X <= 16) go(std::integral_constant<int, 16>{});
+    else if (X <= 32) go(std::integral_constant<int, 32>{});
+    else go(std::integral_constant<int, 64>{});
 }
 
-__global__ void __launch_bounds__(kRowThreads *kRowsPerBlock)
+template <int T>
+__global__ void __launch_bounds__(kRowThreads)
     model_kernel(const __grid_constant__ WaveGeo geo, const float *__restrict__ v, float *__restrict__ m, float s)
 {
     const int r = geo.r, X = geo.nx + 2 * r;
     const int64_t Y = geo.ny + 2 * r, rows = Y * (geo.nz + 2 * r);
-    for (int64_t row = (int64_t)blockIdx.x * kRowsPerBlock + threadIdx.y; row < rows;
-         row += (int64_t)gridDim.x * kRowsPerBlock) {
+    for (int64_t row = (int64_t)blockIdx.x * (kRowThreads / T) + threadIdx.y; row < rows;
+         row += (int64_t)gridDim.x * (kRowThreads / T)) {
         const int64_t zz = row / Y, yy = row - zz * Y, y = yy - r, z = zz - r;
         const bool inside = y >= 0 && y < geo.ny && z >= 0 && z < geo.nz;
         const float *vr = v + (z * geo.ny + y) * geo.nx;
         float *mr = m + zz * geo.pz + yy * geo.py;
-        for (int xx = threadIdx.x; xx < X; xx += kRowThreads) {
+        for (int xx = threadIdx.x; xx < X; xx += T) {
             const int x = xx - r;
             float val = 0.f;
             if (inside && x >= 0 && x < geo.nx) {
@@ -708,17 +720,18 @@ __device__ __forceinline__ double divide_by_float(double g, float m)
     return g / (double)m;
 }
 
-__global__ void __launch_bounds__(kRowThreads *kRowsPerBlock)
+template <int T>
+__global__ void __launch_bounds__(kRowThreads)
     divide_m_kernel(const __grid_constant__ WaveGeo geo, const float *__restrict__ m, double *__restrict__ grad)
 {
     const int r = geo.r;
     const int64_t rows = (int64_t)geo.ny * geo.nz;
-    for (int64_t row = (int64_t)blockIdx.x * kRowsPerBlock + threadIdx.y; row < rows;
-         row += (int64_t)gridDim.x * kRowsPerBlock) {
+    for (int64_t row = (int64_t)blockIdx.x * (kRowThreads / T) + threadIdx.y; row < rows;
+         row += (int64_t)gridDim.x * (kRowThreads / T)) {
         const int64_t z = row / geo.ny, y = row - z * geo.ny;
         double *gr = grad + row * geo.nx;
         const float *mr = m + (z + r) * geo.pz + (y + r) * geo.py + r;
-        for (int x = threadIdx.x; x < geo.nx; x += kRowThreads) gr[x] = divide_by_float(gr[x], mr[x]);
+        for (int x = threadIdx.x; x < geo.nx; x += T) gr[x] = divide_by_float(gr[x], mr[x]);
     }
 }
 
@@ -994,8 +1007,9 @@ cudaError_t launch_model_from_velocity(const WaveGeo &g, const float *v, float *
                                        cudaStream_t st)
 {
     const float s = (dt * dt) / (h * h);
-    model_kernel<<<row_blocks((int64_t)(g.ny + 2 * g.r) * (g.nz + 2 * g.r)), dim3(kRowThreads, kRowsPerBlock), 0, st>>>(
-        g, v, m, s);
+    launch_rows(g.nx + 2 * g.r, (int64_t)(g.ny + 2 * g.r) * (g.nz + 2 * g.r), [&](auto t, int blocks, dim3 block) {
+        model_kernel<decltype(t)::value><<<blocks, block, 0, st>>>(g, v, m, s);
+    });
     return cudaGetLastError();
 }
 
@@ -1009,7 +1023,9 @@ cudaError_t launch_grad_to_velocity(const double *gm, const float *v, double *gv
 
 cudaError_t launch_grad_divide_m(const WaveGeo &g, const float *m, double *grad, cudaStream_t st)
 {
-    divide_m_kernel<<<row_blocks((int64_t)g.ny * g.nz), dim3(kRowThreads, kRowsPerBlock), 0, st>>>(g, m, grad);
+    launch_rows(g.nx, (int64_t)g.ny * g.nz, [&](auto t, int blocks, dim3 block) {
+        divide_m_kernel<decltype(t)::value><<<blocks, block, 0, st>>>(g, m, grad);
+    });
     return cudaGetLastError();
 }
 
